@@ -865,7 +865,7 @@ def trace_summary(args):
         st = spchol.stats(h)
         tr = spchol.trace_get(h, 0).astype(np.int64)
         spchol.destroy(h)
-        ns, nt, nu, nsub = sc["ns"], sc["n_trsm"], sc["n_u"], sc["n_sub"]
+        ns, nt, nu, nsub = sc["ns"], sc["n_trsm"], sc["n_u"], st["n_subtrees"]
         ran = tr[:, 1] > tr[:, 0]
         t0 = tr[ran, 0].min()
         t1 = tr[ran, 1].max()

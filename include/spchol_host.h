@@ -57,6 +57,14 @@ enum {
 int spchol_plan_build(int64_t n, const int64_t* colptr, const int32_t* rowind, const int64_t* perm,
                       const spchol_options* opt, spchol_plan_t* out);
 
+/*
+ * Cut the subtree tasks of more than max_steps steps (diagonal tasks,
+ * panel-solve tiles and update tiles) into the maximal subtrees inside them
+ * that stay within it, as spchol_analyze does for its launch; max_steps < 0:
+ * with spchol_analyze's own limit.  Returns 0 or -1.
+ */
+int spchol_plan_split_subtrees(spchol_plan_t p, int64_t max_steps);
+
 /* Length of array `what`, or -1 for an unknown id. */
 int64_t spchol_plan_len(spchol_plan_t p, int what);
 

@@ -368,6 +368,18 @@ bool build_tensor_maps(spchol_handle_t h, std::vector<CUtensorMap>& maps) {
 int setup_device(spchol_handle_t h) {
   Plan& P = h->plan;
   const int ns = P.ns;
+  // the subtree tasks run by single warps (FP64 DFMA mode) in a launch of
+  // their own before the task loop, when every subtree task qualifies and the
+  // subtrees hold a good part of the work (a batch of small matrices: 30-47 %;
+  // a single large matrix: under 6 %, where the launch ahead of the task loop
+  // costs more than the warps gain; with some subtree tasks left to the CTAs
+  // the task loop would wait for that launch and then run them)
+  const bool warp_sub = mma_mode_of(h->opt.precision) == 0 && !P.params.fanin && P.n_sub > 0 &&
+                        (int32_t)P.wsub.size() == P.n_sub && P.sub_work_frac >= 0.2 &&
+                        h->opt.fault_inject == 0;
+  // the others run on CTAs, none longer than a fair share of the launch (the
+  // fault injection withholds the flop budget's task of the root)
+  if (!warp_sub && h->opt.fault_inject == 0) split_subtrees(P, subtree_step_budget(P));
   Arena& A = h->arena;
   auto r32 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int32_t)); };
   auto r64 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int64_t)); };
@@ -383,15 +395,6 @@ int setup_device(spchol_handle_t h) {
   // seeds: every subtree task, and the panels outside subtrees with no
   // incoming update
   std::vector<int32_t> fseeds;
-  // the subtree tasks run by single warps (FP64 DFMA mode) in a launch of
-  // their own before the task loop, when every subtree task qualifies and the
-  // subtrees hold a good part of the work (a batch of small matrices: 30-47 %;
-  // a single large matrix: under 6 %, where the launch ahead of the task loop
-  // costs more than the warps gain; with some subtree tasks left to the CTAs
-  // the task loop would wait for that launch and then run them)
-  const bool warp_sub = mma_mode_of(h->opt.precision) == 0 && !P.params.fanin && P.n_sub > 0 &&
-                        (int32_t)P.wsub.size() == P.n_sub && P.sub_work_frac >= 0.2 &&
-                        h->opt.fault_inject == 0;
   std::vector<char> by_warp(P.n_sub, 0);
   if (warp_sub)
     for (int32_t k : P.wsub) by_warp[k] = 1;

@@ -175,6 +175,12 @@ int spchol_plan_build(int64_t n, const int64_t* colptr, const int32_t* rowind, c
   return 0;
 }
 
+int spchol_plan_split_subtrees(spchol_plan_t p, int64_t max_steps) {
+  if (!p) return -1;
+  split_subtrees(p->plan, max_steps >= 0 ? max_steps : subtree_step_budget(p->plan));
+  return 0;
+}
+
 int64_t spchol_plan_len(spchol_plan_t p, int what) {
   if (!p) return -1;
   const Plan& P = p->plan;

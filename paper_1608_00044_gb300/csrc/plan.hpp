@@ -232,4 +232,33 @@ struct PlanError {
 int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const int64_t* perm,
                const PlanParams& params, Plan& plan, PlanError& err);
 
+// Replaces every subtree task of more than max_steps steps (a step: a diagonal
+// task, a panel-solve tile or an update tile) by the maximal subtrees inside it
+// that stay within max_steps; the panels above those become tasks of their
+// own.  Not after the warp-level launches have been laid out (Plan::wsub).
+void split_subtrees(Plan& plan, int64_t max_steps);
+
+// The GPU launch's max_steps: a CTA's average share of all steps (152 SMs x 5
+// resident CTAs) over kSubtreeShare.  A subtree task runs its steps one after
+// another, so one that holds more than the average share of the whole
+// factorization outlasts everything else: the 1e6-flop budget alone left the
+// 31 x 34 x 29 Laplacian with 128 tasks of up to 2633 steps (13 of its 19.6
+// ms) against an average share of 645.  Measured factorization times (ms) by
+// kSubtreeShare, "none" the flop budget alone:
+//                          none     2      3      4      8     16
+//   64^2 (FP64)            0.556  0.523  0.527  0.531  0.531  0.526
+//   181 x 203              2.08   1.73   1.78   1.81   1.86   1.97
+//   31 x 34 x 29          19.5   11.29  10.85  10.93  10.92  10.97
+//   40^3                  37.5   33.8   33.4   33.1   33.1   33.2
+//   40^3, FP32 panels     19.1   15.8   15.5   15.0   14.9   15.0
+//   27-point 48^3, FP32   17.94  17.94  17.99  18.04  18.18  18.30
+//   27-point 35x31x38, TF32X3 7.15 6.66  6.68   6.72   7.00   7.10
+// (the subtrees of 50^3 and 64^3 are within it from 4 and 6 on).
+constexpr int kSubtreeShare = 3;
+inline int64_t subtree_step_budget(const Plan& P) {
+  int64_t total = 0;
+  for (int32_t s = 0; s < P.ns; ++s) total += 1 + P.ntrsm[s] + P.nu[s];
+  return total / (152 * 5 * kSubtreeShare);
+}
+
 }  // namespace spchol

@@ -786,4 +786,48 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
   return 0;
 }
 
+void split_subtrees(Plan& P, int64_t max_steps) {
+  if (P.n_sub == 0) return;
+  const int32_t ns = P.ns;
+  // steps of each panel's descendants inside its subtree task, itself included,
+  // and the first of them (children precede their parents)
+  std::vector<int64_t> steps(ns, 0);
+  std::vector<int32_t> first(ns);
+  for (int32_t k = 0; k < P.n_sub; ++k) {
+    for (int32_t s = P.sub_lo[k]; s <= P.sub_hi[k]; ++s) first[s] = s;
+    for (int32_t s = P.sub_lo[k]; s <= P.sub_hi[k]; ++s) {
+      steps[s] += 1 + P.ntrsm[s] + P.nu[s];
+      if (s < P.sub_hi[k]) {
+        const int32_t p = P.parent[s];
+        steps[p] += steps[s];
+        first[p] = std::min(first[p], first[s]);
+      }
+    }
+  }
+  std::vector<int32_t> lo, hi, in(ns, -1);
+  for (int32_t k = 0; k < P.n_sub; ++k)
+    for (int32_t s = P.sub_lo[k]; s <= P.sub_hi[k]; ++s) {
+      const bool root = steps[s] <= max_steps && (s == P.sub_hi[k] || steps[P.parent[s]] > max_steps);
+      if (root && s > first[s]) {  // a subtree of one panel gains nothing
+        for (int32_t q = first[s]; q <= s; ++q) in[q] = (int32_t)lo.size();
+        lo.push_back(first[s]);
+        hi.push_back(s);
+      }
+    }
+  for (int32_t s = 0; s < ns; ++s)
+    if (P.in_sub[s] >= 0 && in[s] < 0) {  // its own tasks are scheduled now
+      P.n_factor_tasks += 1 + P.ntrsm[s] + P.nu[s];
+      P.n_hi_tasks += 1 + P.ntrsm[s] + P.nu_hi[s];
+    }
+  const int32_t more = (int32_t)lo.size() - P.n_sub;
+  P.n_sub += more;
+  P.n_task_ids += more;
+  P.n_factor_tasks += more;
+  P.n_hi_tasks += more;
+  P.sub_lo.swap(lo);
+  P.sub_hi.swap(hi);
+  P.in_sub.swap(in);
+  P.wsub.clear();  // the warp-level launches take the tasks as they were
+}
+
 }  // namespace spchol

@@ -444,3 +444,43 @@ def test_w_panel_solve_protocol(name, W, depth):
         rc, X, _ = P.simulate(A.values, B, seed=seed)
         assert rc == 0
         np.testing.assert_allclose(X, Xo, rtol=1e-11, atol=1e-13)
+
+
+@pytest.mark.parametrize("name,W,max_steps", [("lap3d_20", 8, 0), ("lap3d_20", 16, 7), ("diff3d_9", 64, 5),
+                                              ("lap2d_64", 16, 20), ("lap2d_64", 16, 10**9), ("lap3d_20", 64, -1)])
+def test_split_subtrees_are_maximal_and_run_the_protocol(name, W, max_steps):
+    """Subtree tasks cut at max_steps steps: whole subtrees inside the old
+    tasks, within the limit, maximal, the scheduled tasks counted again -- and
+    the simulator runs the cut plan to the uncut plan's factor."""
+    A, perm, b = gridgen.workload(name)
+    P, Q = _plan(A, perm, max_width=W), _plan(A, perm, max_width=W)
+    Q.split_subtrees(max_steps)
+    par, ntr, nu, nuhi = P.get(hp.PARENT), P.get(hp.NTRSM), P.get(hp.NU), P.get(hp.NUHI)
+    ns, own = len(par), 1 + ntr + nu
+    if max_steps < 0:
+        max_steps = int(own.sum()) // (152 * 5 * 3)
+    old = np.full(ns, -1)
+    for k, (a, r) in enumerate(zip(P.get(hp.SUBLO), P.get(hp.SUBHI))):
+        old[a:r + 1] = k
+    steps, size = own.copy(), np.ones(ns, int)
+    for s in range(ns):
+        if par[s] >= 0 and old[par[s]] >= 0:
+            steps[par[s]] += steps[s]
+            size[par[s]] += size[s]
+    lo, hi = Q.get(hp.SUBLO), Q.get(hp.SUBHI)
+    want = [(s - size[s] + 1, s) for s in range(ns) if old[s] >= 0 and steps[s] <= max_steps and size[s] > 1
+            and (par[s] < 0 or old[par[s]] < 0 or steps[par[s]] > max_steps)]
+    assert list(zip(lo, hi)) == want
+    out = np.ones(ns, bool)
+    for a, r in want:
+        out[a:r + 1] = False
+    sc = Q.scalars()
+    assert sc["n_sub"] == len(want)
+    assert sc["factor_tasks"] == len(want) + int(own[out].sum())
+    assert sc["n_hi_tasks"] == len(want) + int((1 + ntr + nuhi)[out].sum())
+    rc0, X0, pool0 = P.simulate(A.values, b, seed=1, want_pool=True)
+    rc, X, pool = Q.simulate(A.values, b, seed=1, want_pool=True)
+    assert rc0 == 0 and rc == 0
+    # the order of the sums alone differs: at most a few hundred roundings of the largest entry
+    assert np.abs(pool - pool0).max() <= 1e-13 * np.abs(pool0).max()
+    assert oracle.berr(A, X, b) <= 1e-14
