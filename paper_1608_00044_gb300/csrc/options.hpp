@@ -62,6 +62,8 @@ inline PlanParams params_from(const spchol_options& o) {
     p.slice_fp64 = true;
   }
   p.trsm_rows = kTrsmTileRows;
+  if (o.precision != SPCHOL_FP64) p.level_trsm = 0.3;
+  if (o.precision == SPCHOL_FP32) p.level_tiles = 1.0;
   p.fifo = o.sched == 1;
   p.solve_rows = o.solve_tile_rows > 0 ? o.solve_tile_rows : kSolveTileRows;
   p.w_depth = o.solve_w_depth > 0 ? o.solve_w_depth : o.solve_w_depth == 0 ? kWDepth : 0;

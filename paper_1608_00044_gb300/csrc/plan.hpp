@@ -27,11 +27,33 @@ struct PlanParams {
   int trsm_rows = 128;   // rows per panel-solve tile
   int solve_rows = 128;  // rows per triangular-solve tile
   // Panels within top_depth of the root of the panel etree (the chains of the
-  // top separators: the critical path) get smaller tiles, so that each step of
-  // the chain spreads over more CTAs.
+  // top separators: the critical path): their update tiles into the etree
+  // parent go ahead of the others, and their solve tiles are shorter.
   int top_depth = 128;
-  int top_tile_rows = 16;
-  int top_trsm_rows = 16;
+  // Rows per update tile: the panels of one level (distance to the root) take
+  // the largest of tile_rows, 32 and 16 that still gives the level level_tiles
+  // tiles per resident CTA of the GPU (kPlanCtas); rows per panel-solve tile:
+  // of trsm_rows, 32 and 16, level_trsm tiles.  A level with fewer is on the
+  // critical path and its tiles have to spread; one with more only pays each
+  // tile's claim, staging and publishing.  level_tiles 0: by the size of the
+  // problem (FP64 tiles), 8 (flops / 2.4e10)^0.4 within 4 .. 32.  Measured, ms
+  // of the FP64 factorization by level_tiles (with 16 rows within 128 levels of
+  // the root and tile_rows below, the rule before: 10.6, 20.5, 33.2, 76.4,
+  // 102.7 and 387.2):
+  //                 4      6      8      12     16     24
+  //   31 x 34 x 29  9.81   9.54   9.91  10.49  10.71
+  //   33 x 41 x 37 19.03  18.25  18.32  18.98  19.92
+  //   40^3         30.4   29.3   28.8   29.7   30.7
+  //   27-pt 48^3   78.1   77.0   76.3   75.0   74.6
+  //   50^3         98.0   97.8   96.8   94.9   95.8
+  //   64^3        390.6  390.6  390.0  388.3  386.9
+  // FP32 tiles are 5 us of arithmetic to 5 us of the rest and want fewer (27-pt
+  // 48^3 by 0.5 / 1 / 2 / 4 / 8: 12.58 / 12.48 / 12.50 / 12.60 / 13.03 ms,
+  // 17.9 before; 40^3 9.7 up to 4, 15.7 before), as do the panel-solve tiles
+  // beside tensor-core updates (64^3 FP64_TC by 0.3 / 1 / 3: 152.3 / 155.1 /
+  // 159.0 ms).
+  double level_tiles = 0.0;
+  double level_trsm = 1.0;
   int top_solve_rows = 32;  // rows per triangular-solve tile of those panels
   // Tensor-core update tiles: source panels at least tc_min_width wide (0 =
   // none) use tc_tile_rows-row tiles (one MMA M-tile) on the tensor cores.
@@ -59,6 +81,9 @@ struct PlanParams {
   // need no diagonal task on the chain: see Plan::woff.
   int w_depth = 0;
 };
+
+// Resident CTAs of the factorization the plan is laid out for: 152 SMs x 5.
+constexpr int kPlanCtas = 152 * 5;
 
 // Widest panel of a subtree task that runs on one warp (Plan::wsub).
 constexpr int kWarpSubW = 32;
@@ -238,8 +263,8 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
 // own.  Not after the warp-level launches have been laid out (Plan::wsub).
 void split_subtrees(Plan& plan, int64_t max_steps);
 
-// The GPU launch's max_steps: a CTA's average share of all steps (152 SMs x 5
-// resident CTAs) over kSubtreeShare.  A subtree task runs its steps one after
+// The GPU launch's max_steps: a CTA's average share of all steps (kPlanCtas)
+// over kSubtreeShare.  A subtree task runs its steps one after
 // another, so one that holds more than the average share of the whole
 // factorization outlasts everything else: the 1e6-flop budget alone left the
 // 31 x 34 x 29 Laplacian with 128 tasks of up to 2633 steps (13 of its 19.6
@@ -258,7 +283,7 @@ constexpr int kSubtreeShare = 3;
 inline int64_t subtree_step_budget(const Plan& P) {
   int64_t total = 0;
   for (int32_t s = 0; s < P.ns; ++s) total += 1 + P.ntrsm[s] + P.nu[s];
-  return total / (152 * 5 * kSubtreeShare);
+  return total / (kPlanCtas * kSubtreeShare);
 }
 
 }  // namespace spchol

@@ -2,6 +2,7 @@
 // column counts, supernodes, relaxed amalgamation, width cap, row structures,
 // storage layout and the task graph.
 #include <algorithm>
+#include <cmath>
 #include <iterator>
 #include <cstring>
 #include <numeric>
@@ -386,16 +387,45 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
   P.trsm_sn.clear();
   P.ut.clear();
   P.n_rel = 0;
+  // ---- rows per update and panel-solve tile, level by level (PlanParams::level_tiles)
+  std::vector<int32_t> upd_rows, solve_rows;
+  {
+    const int32_t levels = ns == 0 ? 0 : *std::max_element(depth.begin(), depth.end()) + 1;
+    const int32_t ur[3] = {prm.tile_rows, std::min(32, prm.tile_rows), std::min(16, prm.tile_rows)};
+    const int32_t tr[3] = {prm.trsm_rows, std::min(32, prm.trsm_rows), std::min(16, prm.trsm_rows)};
+    std::vector<int64_t> nu(2 * (size_t)levels, 0), nt(2 * (size_t)levels, 0);
+    for (int32_t s = 0; s < ns; ++s) {
+      const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
+      const int32_t* R = P.rows.data() + P.rowoff[s];
+      int64_t* u = nu.data() + 2 * (size_t)depth[s];
+      int64_t* t = nt.data() + 2 * (size_t)depth[s];
+      for (int q = 0; q < 2; ++q) t[q] += (r - w + tr[q] - 1) / tr[q];
+      for (int32_t a = w; a < r;) {
+        for (int q = 0; q < 2; ++q) u[q] += (r - a + ur[q] - 1) / ur[q];
+        a = (int32_t)(std::lower_bound(R + a, R + r, P.fcol[P.snode_of[R[a]] + 1]) - R);
+      }
+    }
+    // FP64 tiles: more of them per CTA on the larger problems (see there)
+    double share = prm.level_tiles;
+    if (share <= 0.0) share = std::min(std::max(8.0 * std::pow(P.flops / 2.4e10, 0.4), 4.0), 32.0);
+    upd_rows.resize(levels);
+    solve_rows.resize(levels);
+    for (int32_t d = 0; d < levels; ++d) {
+      upd_rows[d] = ur[nu[2 * d] >= share * kPlanCtas ? 0 : nu[2 * d + 1] >= share * kPlanCtas ? 1 : 2];
+      solve_rows[d] = tr[nt[2 * d] >= prm.level_trsm * kPlanCtas ? 0 : nt[2 * d + 1] >= prm.level_trsm * kPlanCtas ? 1 : 2];
+    }
+  }
+  auto update_rows = [&](int32_t s) {
+    const bool tc = prm.tc_min_width > 0 && P.fcol[s + 1] - P.fcol[s] >= prm.tc_min_width;
+    return std::max(1, tc ? prm.tc_tile_rows : upd_rows[depth[s]]);
+  };
   {
     // the tile count first (the same walk), so that the tile list is built in
     // place: millions of tiles on the large grids
     int64_t nt = 0, ntr = 0;
     for (int32_t s = 0; s < ns; ++s) {
       const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
-      const bool top = depth[s] < prm.top_depth;
-      const bool tc = prm.tc_min_width > 0 && w >= prm.tc_min_width;
-      const int TU = std::max(1, tc ? prm.tc_tile_rows : top ? std::min(prm.top_tile_rows, prm.tile_rows) : prm.tile_rows);
-      const int TR = std::max(1, top ? std::min(prm.top_trsm_rows, prm.trsm_rows) : prm.trsm_rows);
+      const int TU = update_rows(s), TR = std::max(1, solve_rows[depth[s]]);
       ntr += (r - w + TR - 1) / TR;
       const int32_t* R = P.rows.data() + P.rowoff[s];
       for (int32_t a = w; a < r;) {
@@ -413,9 +443,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
     const int32_t nb = r - w;
     const bool top = depth[s] < prm.top_depth;
-    const bool tc = prm.tc_min_width > 0 && w >= prm.tc_min_width;
-    const int TU = std::max(1, tc ? prm.tc_tile_rows : top ? std::min(prm.top_tile_rows, prm.tile_rows) : prm.tile_rows);
-    const int TR = std::max(1, top ? std::min(prm.top_trsm_rows, prm.trsm_rows) : prm.trsm_rows);
+    const int TU = update_rows(s), TR = std::max(1, solve_rows[depth[s]]);
     P.trsm_rows[s] = TR;
     P.trsm_first[s] = (int32_t)P.trsm_sn.size();
     P.ntrsm[s] = (nb + TR - 1) / TR;
