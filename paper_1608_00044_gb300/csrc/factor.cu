@@ -47,20 +47,28 @@ __device__ __forceinline__ T* panel_ptr(const FactorArgs& a, int s) {
 }
 
 // ---------------------------------------------------------------- POTRF(s)
-// Cholesky of the w x w diagonal block in shared memory (Algorithm 1), taken
-// right-looking in the square-root-free form A = M D M^T, one barrier per
-// column, then L = M D^{1/2}.  Step j: warps 0..6 form the multipliers
-// m_ij = a_ij / d_j (into a double-buffered vector), write column j - 1 of M
-// back in place, and apply the rank-1 update a_ik -= m_ij a_kj of the
-// trailing triangle; meanwhile warp 7 already updates d_{j+1} and forms
-// 1 / d_{j+1} (look-ahead).  The serial chain from one column to the next is
-// a multiply, an FMA and a reciprocal; the square roots come after the loop,
-// all columns at once.  The update is enumerated by the pair index p of the
-// trailing triangle in column-major order from its bottom-right corner, so
-// that p < m (m + 1) / 2 is exactly the triangle of order m and consecutive p
-// touch consecutive rows; the pairs are decoded once into a table.
-constexpr int kPivotWarp = 7;
-constexpr int kUpdWarps = 7;
+// Cholesky of the w x w diagonal block in shared memory (Algorithm 1),
+// right-looking, two columns and one barrier per step.  Step c: the pivot warp
+// finishes columns c and c + 1 (rows c .. c + 31; a second warp the rows
+// below them) -- subtracts columns c - 2 and c - 1 from them and scales them --
+// while the update warps subtract columns c - 2 and c - 1 from the columns
+// beyond.  What bounds it: a warp-wide FP64 instruction holds one of the SM's
+// four FP64 pipes for 64 clocks whatever its active lanes, warps issue in
+// order, and a warp whose lanes are all predicated off still takes its turn.
+// So the pivots' reciprocal square roots run on the integer pipe (seven FP64
+// instructions per pair of columns are left on the chain), the update warps
+// leave the pivot warps' sub-partitions to them as far as they can (warp 3
+// comes last), and a warp branches around the pairs it has none of.  A w = 64
+// block alone on an SM (clocks, w = 32 in parentheses): 75,800 (32,600) one
+// column per step with the square root in FP64, 59,600 (24,800) this way; the
+// chain alone is 49,700, the updates alone 39,700.
+// The trailing entries are enumerated by the pair index p of the triangle in
+// column-major order from its bottom-right corner, so that p < m (m + 1) / 2
+// is exactly the triangle of order m and consecutive p touch consecutive rows;
+// each thread decodes its first pairs once.
+constexpr int kPivotWarp = 7;   // and kPivotWarp - 1: the rows from c + 32 on
+constexpr int kUpdWarps = 6;    // warps 0, 1, 2, 4, 5 and 3
+constexpr int kPairRegs = 10;   // pairs a thread keeps decoded: 10 x 192 >= 60 x 61 / 2 (w = 64)
 
 __device__ __forceinline__ void tri_pair(int p, int& ei, int& ek) {
   int e = (int)((sqrtf((float)(8 * p + 1)) - 1.0f) * 0.5f);
@@ -86,98 +94,276 @@ __device__ __forceinline__ double pivot_recip(double d) {
   return 1.0 / d;
 }
 
+// d > 0 on the integer pipe (false for a NaN, as the comparison).
+__device__ __forceinline__ bool pivot_positive(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b <= 0x7FF0000000000000ll;
+}
+
+// 1 / sqrt(d) for the pivot d > 0, in integers: one step of third order,
+// y (1 + e / 2 + 3 e^2 / 8) with e = 1 - d y^2, from the single-precision
+// approximate reciprocal square root y of d cut to single precision (|e| <
+// 2^-20: the remainder 5/16 e^3 is below 2^-61).  With d = M 2^(E - 52) and y =
+// Y 2^(F - 23), d y^2 = M Y^2 2^(E + 2F - 98), so e is the low part of -M Y^2
+// taken from its bit 32 on (its high part is the power of two next to it), in
+// units of 2^(E + 2F - 66); everything below is kept to 2^-57 and the result
+// rounded to nearest (largest error seen over 1.5e8 values: 0.51 units of
+// 2^-52 of a mantissa near 1).  Outside |exponent| < 120, the square root and
+// the division.
+__device__ __forceinline__ double pivot_rsqrt(double d) {
+  const int hi = __double2hiint(d);
+  const unsigned lo = (unsigned)__double2loint(d);
+  if ((unsigned)(hi - (903 << 20)) < (unsigned)(240 << 20)) {
+    float f;
+    asm("rsqrt.approx.ftz.f32 %0, %1;"
+        : "=f"(f)
+        : "f"(__int_as_float(((hi - (896 << 20)) << 3) | (int)(lo >> 29))));
+    const unsigned fb = __float_as_uint(f);
+    const unsigned Y = (fb & 0x7fffffu) | 0x800000u;
+    const int fe = (int)(fb >> 23);
+    const unsigned long long Q = (unsigned long long)Y * Y;
+    const unsigned mh = (hi & 0xFFFFF) | 0x100000, qh = (unsigned)(Q >> 32), ql = (unsigned)Q;
+    unsigned long long t = (unsigned long long)mh * ql + __umulhi(lo, ql);
+    t += (unsigned long long)lo * qh;
+    t += (unsigned long long)(mh * qh) << 32;
+    const long long e = (-(long long)t) >> (1283 - (hi >> 20) - 2 * fe);  // units of 2^-60
+    const int eh = (int)(e >> 20);
+    const long long c = (e >> 1) + (((long long)eh * eh * 3) >> 23);
+    const unsigned long long y = ((unsigned long long)Y << 39) + (((long long)Y * c) >> 21);
+    const int lz = __clzll((long long)y);
+    const unsigned long long yn = y << lz;
+    return __longlong_as_double(((long long)(fe + 896 - lz) << 52) + (long long)((yn >> 11) + ((yn >> 10) & 1)));
+  }
+  return 1.0 / sqrt(d);
+}
+
+// Columns c and c + 1 of rows i = row(lane) from columns c - 2 and c - 1 (c >
+// 0): the entries before scaling.
+__device__ __forceinline__ void pivot_load(const double* sm, int w, int c, int i, double& v2, double& v3) {
+  const double* c2 = sm + c * w;
+  const bool rv = i < w, two = c + 1 < w;
+  v2 = rv ? c2[i] : 0.0;
+  v3 = two && rv && i > c ? c2[w + i] : 0.0;
+  if (c > 0) {
+    const double *c1 = c2 - w, *c0 = c1 - w;
+    const double a0 = rv ? c0[i] : 0.0, a1 = rv ? c1[i] : 0.0;
+    const double e0 = two ? c0[c + 1] : 0.0, e1 = two ? c1[c + 1] : 0.0;
+    v2 = fma(-a1, c1[c], fma(-a0, c0[c], v2));
+    v3 = fma(-a1, e1, fma(-a0, e0, v3));
+  }
+}
+
+// The pivot warps finish columns c and c + 1.  MAIN: rows c .. c + 31 and
+// 1 / l_cc, 1 / l_c+1,c+1 in xd; else the rows from c + 32 on, lanes 30 and 31
+// of the first pass repeating rows c and c + 1 for the pivots.  The main warp
+// overwrites those two rows only after the other one has read them (both = the
+// other one takes part).  A pivot that is not positive is reported; the
+// columns after it are not meaningful and are not used.
+template <bool MAIN>
+__device__ __forceinline__ void pivot_pair(const FactorArgs& a, double* sm, double* xd, int w, int c, int f,
+                                           bool both) {
+  const int lane = threadIdx.x & 31;
+  const bool two = c + 1 < w;
+  constexpr int kL = MAIN ? 0 : 30;  // the lanes that hold rows c and c + 1
+  int i = MAIN ? c + lane : lane < 30 ? c + 32 + lane : c + lane - 30;
+  double v2, v3;
+  pivot_load(sm, w, c, i, v2, v3);
+  if (!MAIN) {
+    __syncwarp();
+    asm volatile("bar.arrive 1, 64;" ::: "memory");
+  }
+  const double d2 = __shfl_sync(0xffffffffu, v2, kL);
+  const double r2 = pivot_rsqrt(d2);
+  double x2 = v2 * r2, x3 = 0.0, r3 = 0.0, d3 = 1.0;
+  const double k32 = __shfl_sync(0xffffffffu, x2, kL + 1);
+  if (two) {
+    v3 = fma(-x2, k32, v3);
+    d3 = __shfl_sync(0xffffffffu, v3, kL + 1);
+    r3 = pivot_rsqrt(d3);
+    x3 = v3 * r3;
+  }
+  if (MAIN) {
+    if (both) asm volatile("bar.sync 1, 64;" ::: "memory");
+    if (lane == 0) {
+      xd[c] = r2;
+      if (two) xd[c + 1] = r3;
+      if (!pivot_positive(d2)) atomicMin(&a.ctrl[kInfo], f + c + 1);
+      if (!pivot_positive(d3)) atomicMin(&a.ctrl[kInfo], f + c + 2);
+    }
+  }
+  double* c2 = sm + c * w;
+  if (MAIN || lane < 30) {
+    if (i < w) {
+      c2[i] = x2;
+      if (two && i > c) c2[w + i] = x3;
+    }
+  }
+  if (!MAIN) {
+    for (i = c + 62 + lane; i - lane < w; i += 32) {
+      pivot_load(sm, w, c, i, v2, v3);
+      x2 = v2 * r2;
+      if (i < w) {
+        c2[i] = x2;
+        if (two) c2[w + i] = fma(-x2, k32, v3) * r3;
+      }
+    }
+  }
+}
+
+// The update warps subtract columns c - 2 and c - 1 from one trailing entry.
+__device__ __forceinline__ void potrf_update(double* sm, int w, int c, int i, int k) {
+  const double *c0 = sm + (c - 2) * w, *c1 = c0 + w;
+  double* s = sm + i + k * w;
+  *s = fma(-c1[i], c1[k], fma(-c0[i], c0[k], *s));
+}
+
+// X = L11^{-1} for the solves, off the critical path (the panel-solve tiles
+// are already released), by block rows of 8: X_bc = inv(L_bb) (-L_b,: X_:,c).
+// First every 8 x 8 diagonal block's inverse (a warp each), then the rows of
+// L below the diagonal blocks are replaced by G_b = -inv(L_bb) L_b,: (in
+// place: L11 is stored), then block row after block row X_b = G_b X, one
+// barrier each, 8 rows x 4 columns per warp and dot products over the columns
+// k >= c alone.  1600 warp-wide FP64 instructions for w = 64 against 2500 and
+// 9 barriers against 63 for the substitution row by row it replaces.  X[i][c],
+// i > c, lives in the upper triangle at (c, i); the diagonal is xd.
+__device__ void invert_l11(double* sm, const double* xd, int w, double* __restrict__ X) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int li = lane & 7, lc = lane >> 3;
+  const int nb = (w + 7) >> 3;
+  for (int b = warp; b < nb; b += kFactorThreads / 32) {
+    // lane (li, lc): row 8 b + li of columns 8 b + lc and 8 b + lc + 4.  With
+    // the rows scaled by 1 / l_ii first, x_ic = -sum over q of l_iq x_qc
+    const int r0 = 8 * b, i = r0 + li;
+    const bool rv = i < w;
+    const double ri = rv ? xd[i] : 0.0;
+    double x0 = li == lc ? ri : 0.0, x1 = li == lc + 4 ? ri : 0.0;
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const double l = (rv && li > q) ? sm[i + (r0 + q) * w] * ri : 0.0;
+      const double y0 = __shfl_sync(0xffffffffu, x0, (lane & 24) | q);
+      const double y1 = __shfl_sync(0xffffffffu, x1, (lane & 24) | q);
+      x0 = fma(-l, y0, x0);
+      x1 = fma(-l, y1, x1);
+    }
+    __syncwarp();
+    if (rv && li > lc) {
+      sm[(r0 + lc) + i * w] = x0;
+      X[i + (size_t)(r0 + lc) * w] = x0;
+    }
+    if (rv && li > lc + 4) {
+      sm[(r0 + lc + 4) + i * w] = x1;
+      X[i + (size_t)(r0 + lc + 4) * w] = x1;
+    }
+  }
+  __syncthreads();
+  // G_b for all block rows: group t of 4 columns of block row b (2 b of them)
+  for (int g = warp; g < nb * (nb - 1); g += kFactorThreads / 32) {
+    int b = 1, t = g;
+    while (t >= 2 * b) {
+      t -= 2 * b;
+      ++b;
+    }
+    const int r0 = 8 * b, i = r0 + li, c = 4 * t + lc;
+    const bool rv = i < w;
+    const double* lcol = sm + r0 + c * w;
+    double acc = rv ? xd[i] * lcol[li] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const double x = (rv && li > q) ? sm[(r0 + q) + i * w] : 0.0;
+      acc = fma(x, (rv && li > q) ? lcol[q] : 0.0, acc);
+    }
+    __syncwarp();
+    if (rv) sm[i + c * w] = -acc;
+  }
+  __syncthreads();
+  for (int b = 1; b < nb; ++b) {
+    const int r0 = 8 * b, i = r0 + li;
+    const bool rv = i < w;
+    for (int r = 0; 8 * r < 2 * b; ++r) {
+      // long and short columns alternate over the warps
+      const int t = 8 * r + ((r & 1) ? 7 - warp : warp);
+      if (t >= 2 * b) continue;
+      const int c = 4 * t + lc;
+      const double* G = sm + i;
+      const double* Xc = sm + c;
+      double a0 = 0.0, a1 = 0.0;
+      if (rv) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = 4 * t + u;
+          const double x = k < c ? 0.0 : k == c ? xd[c] : Xc[k * w];
+          a0 = fma(G[k * w], x, a0);
+        }
+        int k = 4 * t + 4;
+        for (; k < r0; k += 4) {  // r0 - 4 t is a multiple of 4
+          a0 = fma(G[k * w], Xc[k * w], a0);
+          a1 = fma(G[(k + 1) * w], Xc[(k + 1) * w], a1);
+          a0 = fma(G[(k + 2) * w], Xc[(k + 2) * w], a0);
+          a1 = fma(G[(k + 3) * w], Xc[(k + 3) * w], a1);
+        }
+        a0 += a1;
+        sm[c + i * w] = a0;
+        X[i + (size_t)c * w] = a0;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 template <typename T, bool FAN>
 __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared& sh, bool skip, bool release = true) {
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int f = a.pv.fcol[s], w = a.pv.fcol[s + 1] - f, ld = a.pv.ld[s];
   T* P = panel_ptr<T>(a, s);
-  double* xd = sm + w * w;  // during the loop 1 / d_j; after it r_j = 1 / l_jj (the diagonal of L11^{-1})
-  double* cb = xd + w;      // 2 x w: multipliers of the current step, by parity
-  // pair table: the column index ek of pair p of the trailing triangle (its
-  // row index is p - ek (ek + 1) / 2), decoded once
-  uint8_t* pt = reinterpret_cast<uint8_t*>(cb + 2 * w);
-  const int npair = w * (w - 1) / 2;  // pairs of the largest trailing triangle (step 0)
+  double* xd = sm + w * w;  // 1 / l_jj, the diagonal of L11^{-1}
+  double* X = a.inv + a.invoff[s];
   bool ok = true;
   if (!skip) {
     stage_lower<true>(P, w, ld, sm);  // lower triangle; zeros above (used below for L11^{-1})
-    for (int p = tid; p < npair; p += blockDim.x) {
-      int ei, ek;
-      tri_pair(p, ei, ek);
-      pt[p] = (uint8_t)ek;
-    }
-    if (tid == 0) sh.flag = 0;
-    __syncthreads();
-    if (tid == kPivotWarp * 32) {
-      const double d0 = sm[0];
-      if (d0 > 0.0) {
-        xd[0] = pivot_recip(d0);
-      } else {
-        atomicMin(&a.ctrl[kInfo], f + 1);
-        sh.flag = 1;
+    const int uw = warp == 3 ? kUpdWarps - 1 : warp > 3 ? warp - 1 : warp;  // number among the update warps
+    const int ut = uw * 32 + lane;
+    constexpr int kStep = kUpdWarps * 32;
+    int pair[kPairRegs];  // row << 16 | column
+    if (warp < kPivotWarp - 1 && w > 4) {
+#pragma unroll
+      for (int q = 0; q < kPairRegs; ++q) {
+        int ei, ek;
+        tri_pair(ut + kStep * q, ei, ek);
+        pair[q] = ((w - 1 - ei) << 16) | ((w - 1 - ek) & 0xffff);
       }
     }
     __syncthreads();
-    for (int j = 0; j < w && !sh.flag; ++j) {
-      const double qj = xd[j];
-      if (warp < kUpdWarps) {
-        double* cj = cb + (j & 1) * w;
-        const double* cprev = cb + ((j + 1) & 1) * w;
-        for (int i = j + 1 + tid; i < w; i += kUpdWarps * 32) cj[i] = sm[i + j * w] * qj;
-        if (j > 0)
-          for (int i = j + tid; i < w; i += kUpdWarps * 32) sm[i + (j - 1) * w] = cprev[i];
-        asm volatile("bar.sync 1, %0;" ::"n"(kUpdWarps * 32) : "memory");
-        const int m = w - 1 - j;
-        const int np = m * (m + 1) / 2 - 1;  // all but (j + 1, j + 1), which warp 7 owns
-        const double* aj = sm + j * w;       // column j, not yet divided by d_j
-        constexpr int kStep = kUpdWarps * 32;
-        // two pairs per round, every load issued before the arithmetic: the
-        // pairs are distinct entries, so the rounds' chains overlap
-        for (int p = tid; p < np; p += 2 * kStep) {
-          const int p2 = p + kStep;
-          const int q2 = p2 < np ? p2 : p;
-          const int ek1 = pt[p], ek2 = pt[q2];
-          const int i1 = w - 1 - (p - ek1 * (ek1 + 1) / 2), k1 = w - 1 - ek1;
-          const int i2 = w - 1 - (q2 - ek2 * (ek2 + 1) / 2), k2 = w - 1 - ek2;
-          const double a1 = cj[i1], b1 = aj[k1], s1 = sm[i1 + k1 * w];
-          const double a2 = cj[i2], b2 = aj[k2], s2 = sm[i2 + k2 * w];
-          sm[i1 + k1 * w] = fma(-a1, b1, s1);
-          if (p2 < np) sm[i2 + k2 * w] = fma(-a2, b2, s2);
+    for (int c = 0; c < w; c += 2) {
+      if (warp == kPivotWarp) {
+        pivot_pair<true>(a, sm, xd, w, c, f, w - c > 32);
+      } else if (warp == kPivotWarp - 1) {
+        if (w - c > 32) pivot_pair<false>(a, sm, xd, w, c, f, true);
+      } else if (c > 0) {
+        const int m = w - 2 - c;  // columns c + 2 .. w - 1
+        const int np = m > 0 ? m * (m + 1) / 2 : 0;
+#pragma unroll
+        for (int q = 0; q < kPairRegs; ++q) {
+          if (kStep * q + 32 * uw >= np) break;
+          if (kStep * q + ut < np) potrf_update(sm, w, c, pair[q] >> 16, pair[q] & 0xffff);
         }
-      } else if (lane == 0 && j + 1 < w) {
-        const double a1 = sm[(j + 1) + j * w];
-        const double d = fma(-(a1 * qj), a1, sm[(j + 1) * (w + 1)]);
-        const double q = pivot_recip(d);
-        if (d > 0.0) {
-          sm[(j + 1) * (w + 1)] = d;
-          xd[j + 1] = q;
-        } else {
-          atomicMin(&a.ctrl[kInfo], f + j + 2);
-          sh.flag = 1;
+        for (int p = kStep * kPairRegs + ut; p < np; p += kStep) {  // w > 64
+          int ei, ek;
+          tri_pair(p, ei, ek);
+          potrf_update(sm, w, c, w - 1 - ei, w - 1 - ek);
         }
       }
       __syncthreads();
     }
-    ok = !sh.flag;
-    if (ok) {
-      // L = M D^{1/2}: l_jj = sqrt(d_j) (and r_j = 1 / l_jj for the solves),
-      // then l_ij = m_ij l_jj below the diagonal
-      for (int j = tid; j < w; j += blockDim.x) {
-        const double l = sqrt(sm[j * (w + 1)]);
-        sm[j * (w + 1)] = l;
-        xd[j] = 1.0 / l;
-      }
-      __syncthreads();
-      for (int j = warp; j < w; j += kFactorThreads / 32) {
-        const double l = sm[j * (w + 1)];
-        for (int i = j + 1 + lane; i < w; i += 32) sm[i + j * w] *= l;
-      }
-      __syncthreads();
-    }
+    // a failed pivot, of this block or of any other: its columns are not used
+    if (tid == 0) sh.flag = ld_relaxed(&a.ctrl[kInfo]) != INT_MAX;
     for (int j = warp; j < w; j += kFactorThreads / 32)
       for (int i = j + lane; i < w; i += 32) P[i + (size_t)j * ld] = (T)sm[i + j * w];
+    // the panel-solve tiles scale by 1 / l_jj
+    for (int j = tid; j < w; j += blockDim.x) X[j + (size_t)j * w] = xd[j];
   }
   publish_cta_writes();
+  ok = !skip && !sh.flag;
   if (FAN && release) {  // fan-in mode: a panel-solve tile also waits for its rows' gathers
     for (int k = tid; k < a.ntrsm[s]; k += blockDim.x) {
       const int kt = a.trsm_first[s] + k;
@@ -186,30 +372,7 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   } else if (release) {
     ring2_push_range(rings_of(a), true, a.pv.ns + a.trsm_first[s], a.ntrsm[s], &sh.base);
   }
-  if (!skip && ok) {
-    // L11^{-1} for the solves, off the critical path (the panel-solve tiles are
-    // already released).  X = L11^{-1} by right-looking forward substitution
-    // on all columns at once: after row k of X is final, every row i > k
-    // subtracts l_ik X[k][:]; the row k + 1 is finished (scaled by r_{k+1}) by
-    // the same thread that applies its last update.  X[i][c], i > c, lives in
-    // the zeroed upper triangle at (c, i); the diagonal is xd.
-    for (int k = 0; k < w - 1; ++k) {
-      for (int i = k + 1 + warp; i < w; i += kFactorThreads / 32) {
-        const double lik = sm[i + k * w];
-        const double ri = xd[i];
-        for (int c = lane; c <= k; c += 32) {
-          const double xkc = (c == k) ? xd[k] : sm[c + k * w];
-          double v = fma(-lik, xkc, sm[c + i * w]);
-          if (i == k + 1) v *= ri;
-          sm[c + i * w] = v;
-        }
-      }
-      __syncthreads();
-    }
-    double* X = a.inv + a.invoff[s];
-    for (int j = warp; j < w; j += kFactorThreads / 32)
-      for (int i = j + lane; i < w; i += 32) X[i + (size_t)j * w] = (i == j) ? xd[j] : sm[j + i * w];
-  }
+  if (ok) invert_l11(sm, xd, w, X);
 }
 
 // ---------------------------------------------------------------- FP64 operand slicing
@@ -302,7 +465,8 @@ __device__ void form_w_rows(const FactorArgs& a, int s, int row0, int cnt, doubl
     const int qq = idx & (kTrsmMaxW - 1), c = idx >> 6;
     Ls[qq + kLd * c] = (qq < w && qq > c) ? (ct)ldcg(P + qq + (size_t)c * ld) : ct(0);
   }
-  for (int c = tid; c < w; c += nt) rinv[c] = ct(1) / (ct)ldcg(P + c + (size_t)c * ld);
+  const double* Xd = a.inv + a.invoff[s];
+  for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));
   __syncthreads();
   const int warp = tid >> 5, lane = tid & 31, lr = lane >> 3, lc = lane & 7;
   const int nstrip = (cnt + 3) >> 2;
@@ -364,7 +528,8 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
       const int qq = idx & (kTrsmMaxW - 1), c = idx >> 6;
       Ls[idx] = (qq < w && qq > c) ? (ct)ldcg(P + qq + (size_t)c * ld) : ct(0);
     }
-    for (int c = tid; c < w; c += nt) rinv[c] = ct(1) / (ct)ldcg(P + c + (size_t)c * ld);
+    const double* Xd = a.inv + a.invoff[s];
+    for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));  // written by the diagonal task
     __syncthreads();
     const int nstrip = (cnt + 3) >> 2;
     for (int st = warp; st < nstrip; st += nt >> 5) {
@@ -1402,13 +1567,12 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
 // at every column and step.  A warp-wide FP64 instruction holds the SM's FP64
 // pipe as long whatever its active lanes (the pipe bounds these warps), so
 // each step spreads its entries over the lanes.  Per panel, in postorder:
-//   * the diagonal block in shared memory (leading dimension kWarpLd): each
-//     multiplier, update and pivot is the diagonal task's operation on the
-//     same operands in the same order, so L11 is the same; the lane of row i
-//     forms its multiplier, then the trailing triangle's updates take one
-//     entry per lane and pass, as does the scaling L = M D^{1/2};
-//   * its inverse by the diagonal task's substitution (the same operations
-//     per entry), each step's entries one per lane and pass;
+//   * the diagonal block in shared memory (leading dimension kWarpLd) in the
+//     square-root-free form A = M D M^T: the lane of row i forms its
+//     multiplier, then the trailing triangle's updates take one entry per lane
+//     and pass, as does the scaling L = M D^{1/2};
+//   * its inverse by substitution row by row, each step's entries one per lane
+//     and pass;
 //   * the panel solve by that inverse, l_rc = sum_{k <= c} a_rk X_ck, one
 //     output per lane and pass (the panel-solve tiles of the task loop solve
 //     by substitution instead: they run before the inverse exists);
@@ -1935,10 +2099,8 @@ cudaError_t launch_warp_subtrees(bool fp32, const FactorArgs& a, int grid, cudaS
 }
 
 size_t factor_smem_bytes(int max_w, int mma_mode) {
-  // POTRF: the block, 1 / l_jj, two scaled columns and the 8-bit pair table;
-  // TRSM: L11 with 64-row columns and 1 / l_cc.
-  size_t tri = ((size_t)max_w * max_w + 3 * (size_t)max_w) * sizeof(double) +
-               (((size_t)max_w * (max_w - 1) / 2 + 15) & ~size_t(15));
+  // POTRF: the block and 1 / l_jj; TRSM: L11 with 64-row columns and 1 / l_cc.
+  size_t tri = ((size_t)max_w * max_w + (size_t)max_w) * sizeof(double);
   // (+ 1: the W rows of W panels restage L11 with leading dimension 65)
   if (max_w <= kTrsmMaxW) tri = std::max(tri, (size_t)(kTrsmMaxW + 2) * max_w * sizeof(double));
   if (mma_mode == 3) {

@@ -830,3 +830,44 @@ def test_warp_subtrees_report_a_failed_pivot():
     assert m == 2
     assert spchol.batch_factorize(h, [M.values for M in mats]) == 0
     spchol.destroy(h)
+
+
+@pytest.mark.parametrize("scale", [0, 501, -501])
+@pytest.mark.parametrize("w", [1, 2, 3, 5, 31, 32, 33, 61, 62, 63, 64, 65, 94, 127, 128])
+def test_one_dense_panel_of_every_width(w, scale):
+    # One full matrix is one diagonal task (two columns a step, the rows past
+    # the 32nd by a second warp, blocks of 8 in the inverse), no other task.
+    # Its condition number is below 8, so L and x are within 8 w roundings of
+    # the dense factor's; 2^501 takes the pivots out of the range of the fast
+    # reciprocal square root.  A pivot that is not positive is reported at its
+    # column, the first of two as well.
+    import scipy.sparse as sp
+
+    rng = np.random.default_rng(w)
+    M = rng.uniform(-1.0, 1.0, (w, w))
+    A = (np.eye(w) + (M + M.T) / (4.0 * max(w, 2))) * 2.0 ** scale
+    cp = np.concatenate([[0], np.cumsum(np.arange(w, 0, -1))]).astype(np.int64)
+    ri = np.concatenate([np.arange(j, w) for j in range(w)]).astype(np.int32)
+    lower = lambda S: np.concatenate([S[j:, j] for j in range(w)])
+    b = rng.uniform(-1.0, 1.0, (w, 3))
+    s = spchol.SparseCholesky(w, cp, ri, max_width=128)
+    assert s.stats()["n_supernodes"] == 1
+    assert s.factorize(lower(A)) == 0
+    Lp, Li, Lx, perm = s.export_factor()
+    L = sp.csc_matrix((Lx, Li, Lp), shape=(w, w)).toarray()
+    P = A[np.ix_(perm, perm)]
+    tol = 8 * 8 * w * 2.0 ** -53
+    assert np.abs(L - np.linalg.cholesky(P)).max() <= tol * np.abs(L).max()
+    X = s.solve(b.copy(order="F"))
+    want = np.linalg.solve(A, b)
+    assert np.abs(X - want).max() <= tol * np.abs(want).max()
+    for j in {0, 1, w // 2, w - 1} & set(range(w)):
+        bad = A.copy()
+        bad[perm[j], perm[j]] *= -1.0
+        assert s.factorize(lower(bad)) == j + 1
+    if w > 2:  # two of them: the first
+        bad = A.copy()
+        bad[perm[1], perm[1]] *= -1.0
+        bad[perm[w - 1], perm[w - 1]] *= -1.0
+        assert s.factorize(lower(bad)) == 2
+    s.close()
