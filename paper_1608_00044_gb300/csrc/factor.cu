@@ -33,6 +33,8 @@ struct FactorShared {
   int skip;
   int flag;
   int base;
+  int next;  // a diagonal task this CTA made ready and runs next (-1: none; thread 0)
+  int hold;  // this CTA holds a high-priority slot, or is inside a subtree task: no continuation
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -365,9 +367,10 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   publish_cta_writes();
   ok = !skip && !sh.flag;
   if (FAN && release) {  // fan-in mode: a panel-solve tile also waits for its rows' gathers
+    fence_gpu();
     for (int k = tid; k < a.ntrsm[s]; k += blockDim.x) {
       const int kt = a.trsm_first[s] + k;
-      if (atom_add_acqrel(&a.tdep[kt], -1) == 1) ring2_push_one(rings_of(a), true, a.pv.ns + kt);
+      if (count_down(&a.tdep[kt])) ring2_push_one(rings_of(a), true, a.pv.ns + kt);
     }
   } else if (release) {
     ring2_push_range(rings_of(a), true, a.pv.ns + a.trsm_first[s], a.ntrsm[s], &sh.base);
@@ -620,14 +623,15 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
   }
   publish_cta_writes();
   if (!release) return;  // inside a subtree task: no counters, the same CTA goes on
-  if (tid == 0) sh.flag = (atom_add_acqrel(&a.trsm_left[s], -1) == 1);
+  if (tid == 0) sh.flag = count_down(&a.trsm_left[s]);
   __syncthreads();
   if (sh.flag) {
     const Ring2 q = rings_of(a);
     const int first = a.pv.ns + a.n_trsm + a.u_first[s], nhi = a.nu_hi[s];
     if (a.u_dep) {  // deterministic order: a tile also waits for its predecessor into the same target
+      fence_gpu();
       for (int i = threadIdx.x; i < a.nu[s]; i += blockDim.x)
-        if (atom_add_acqrel(&a.u_dep[a.u_first[s] + i], -1) == 1) ring2_push_one(q, i < nhi, first + i);
+        if (count_down(&a.u_dep[a.u_first[s] + i])) ring2_push_one(q, i < nhi, first + i);
     } else {
       ring2_push_range(q, true, first, nhi, &sh.base);
       ring2_push_range(q, false, first + nhi, a.nu[s] - nhi, &sh.base);
@@ -646,9 +650,16 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
 template <bool FAN>
 __device__ __forceinline__ void target_update_done(const FactorArgs& a, int t, FactorShared& sh, bool release) {
   if constexpr (!FAN) {
-    if (release && threadIdx.x == 0 && atom_add_acqrel(&a.dep_f[t], -1) == 1) ring2_push_one(rings_of(a), true, t);
+    // the diagonal task follows in this CTA, unless it holds a claimed slot
+    // whose task another would then wait for
+    if (release && threadIdx.x == 0 && count_down(&a.dep_f[t])) {
+      if (sh.hold)
+        ring2_push_one(rings_of(a), true, t);
+      else
+        sh.next = t;
+    }
   } else {
-    if (threadIdx.x == 0) sh.flag = release && atom_add_acqrel(&a.dep_f[t], -1) == 1;
+    if (threadIdx.x == 0) sh.flag = release && count_down(&a.dep_f[t]);
     __syncthreads();
     if (sh.flag) {
       const int g0 = a.gat_first[t], g1 = a.gat_first[t + 1];
@@ -1720,6 +1731,7 @@ __device__ void warp_subtree(const FactorArgs& a, int k, double* ws) {
     }
     // update tiles of panel s
     const int32_t* Rs = a.pv.rows + a.pv.rowoff[s];
+    bool any_out = false;
     for (int ui = a.u_first[s]; ui < a.u_first[s] + a.nu[s]; ++ui) {
       const UTask u = a.ut[ui];
       const bool outside = u.t > hi;
@@ -1752,12 +1764,14 @@ __device__ void warp_subtree(const FactorArgs& a, int k, double* ws) {
             *dst -= c0 + c1;
         }
       }
-      if (outside) {  // publish the warp's atomics, then count the tile down on its target
-        __syncwarp();
-        if (lane == 0) {
-          __threadfence();
-          if (atom_add_acqrel(&a.dep_f[u.t], -1) == 1) ring2_push_one(q, true, u.t);
-        }
+      any_out = any_out || outside;
+    }
+    if (any_out) {  // publish the warp's atomics, then count its tiles down on their targets, one per lane
+      __syncwarp();
+      fence_gpu();
+      for (int ui = a.u_first[s] + lane; ui < a.u_first[s] + a.nu[s]; ui += 32) {
+        const int t = a.ut[ui].t;
+        if (t > hi && count_down(&a.dep_f[t])) ring2_push_one(q, true, t);
       }
     }
     __syncwarp();  // the next panel reads what this one's tiles wrote into it
@@ -1782,7 +1796,10 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
   double* smd = reinterpret_cast<double*>(smem_raw);
   const Ring2 q = rings_of(a);
   __shared__ int pend[3];  // claimed, not yet taken ring slots (thread 0)
-  if (threadIdx.x == 0) pend[0] = pend[1] = pend[2] = -1;
+  if (threadIdx.x == 0) {
+    pend[0] = pend[1] = pend[2] = -1;
+    sh.next = -1;
+  }
   // per-CTA task timing (thread 0 only, in shared memory so that no register
   // stays live across the tasks), flushed once at exit: [0..4] busy ns per task
   // type ([3]: tensor-core update tiles, [4]: subtree tasks), [5..9] counts,
@@ -1845,7 +1862,10 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       if (cur_task < 0) {
         const uint64_t t0 = timed ? global_ns() : 0;
         const bool idle = pend[1] < 0 && pend[2] < 0;
-        if (stash >= 0) {  // acquired by the previous claim
+        if (sh.next >= 0) {  // made ready by this CTA's last task
+          sh.task = sh.next;
+          sh.next = -1;
+        } else if (stash >= 0) {  // acquired by the previous claim
           sh.task = stash;
           stash = -1;
           if (deep && idle) ahead = atomicAdd(&q.ctrl[kHead], 2);
@@ -1882,6 +1902,9 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
           cur_skip = sh.skip;
         }
       }
+      // a CTA that holds a high-priority slot takes no continuation: that
+      // slot's task would wait for it
+      sh.hold = cur_task >= 0 || pend[0] >= 0;
       if (cur_task >= 0) {  // the next step of the subtree, then advance the cursor
         const int s = cur_s;
         step_kind = cur_ph;
@@ -1962,8 +1985,8 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       publish_cta_writes();
       if (threadIdx.x == 0) {
         if (o < a.pv.ns) {
-          if (atom_add_acqrel(&a.gdiag[t], -1) == 1) ring2_push_one(rings_of(a), true, t);
-        } else if (atom_add_acqrel(&a.tdep[o - a.pv.ns], -1) == 1) {
+          if (count_down(&a.gdiag[t])) ring2_push_one(rings_of(a), true, t);
+        } else if (count_down(&a.tdep[o - a.pv.ns])) {
           ring2_push_one(rings_of(a), true, o);
         }
       }
@@ -1994,7 +2017,7 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       // (the tile's scatter-adds were published before its own release)
       if (a.u_next && release && threadIdx.x == 0) {
         const int nx = a.u_next[ui];
-        if (nx >= 0 && atom_add_acqrel(&a.u_dep[nx], -1) == 1) {
+        if (nx >= 0 && count_down(&a.u_dep[nx])) {
           const int sx = a.ut[nx].s;
           ring2_push_one(rings_of(a), nx - a.u_first[sx] < a.nu_hi[sx], a.pv.ns + a.n_trsm + nx);
         }

@@ -26,12 +26,17 @@ namespace spchol {
 
 namespace {
 
+constexpr int kWReady = 4;
+
 struct SolveShared {
   int task;
   int flag;
   int base;
   int next;  // continuation: a task this CTA made ready and runs next (-1: none)
   int hold;  // this CTA holds a claimed, still empty ring slot: no continuation
+  int keep;
+  int nw;      // W panels whose last forward tile this task was
+  int wl[kWReady];  // the first of them
 };
 
 template <typename T>
@@ -942,12 +947,14 @@ __device__ void bwd_tile(const SolveArgs& a, int s, int k, double* sm) {
 // Lower the counters cnt[id] of ids list[e] (or e itself when list is null),
 // e in [e0, e1), by one, and push task task0 + id for each that reaches zero
 // (the first one kept as the CTA's continuation if next is given and free).
-// Whole CTA, all threads through the same iterations; each thread issues its
-// decrements in batches of 8 whose round trips overlap, and each warp
-// reserves ring slots for its ready tasks at once (a panel near the root
-// releases thousands of tiles).
+// Whole CTA, all threads through the same iterations, after the barrier that
+// follows what the tasks read; each thread fences once, its decrements go out
+// in batches of 8 whose round trips overlap, and each warp reserves ring slots
+// for its ready tasks at once (a panel near the root releases thousands of
+// tiles).
 __device__ __forceinline__ void release_tiles(const Ring2& q, const int32_t* list, int e0, int e1, int32_t* cnt,
                                               int task0, int* next) {
+  if (e0 + (int)(threadIdx.x & ~31u) < e1) fence_gpu();
   for (int b0 = e0; b0 < e1; b0 += 8 * blockDim.x) {
     int id[8], old[8];
 #pragma unroll
@@ -955,18 +962,23 @@ __device__ __forceinline__ void release_tiles(const Ring2& q, const int32_t* lis
       const int e = b0 + threadIdx.x + u * blockDim.x;
       id[u] = e < e1 ? (list ? list[e] : e) : -1;
     }
-    // acq_rel decrements: each one releases what its thread has observed (the
-    // CTA's writes, ordered before it by the publishing barrier), and the one
-    // that reaches zero acquires every earlier decrement's release, so the
-    // pushed (or kept) task sees all of its producers' writes.
 #pragma unroll
-    for (int u = 0; u < 8; ++u) old[u] = id[u] >= 0 ? atom_add_acqrel(&cnt[id[u]], -1) : 0;
+    for (int u = 0; u < 8; ++u) old[u] = id[u] >= 0 ? atom_add_relaxed(&cnt[id[u]], -1) : 0;
     int ready[8];
+    bool any = false;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       ready[u] = (id[u] >= 0 && old[u] == 1) ? task0 + id[u] : -1;
-      if (ready[u] >= 0 && next != nullptr && atomicCAS(next, -1, ready[u]) == -1) ready[u] = -1;  // kept
+      any = any || ready[u] >= 0;
     }
+    if (any) {
+      fence_gpu();  // acquire what the other decrements signalled
+      if (next != nullptr)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (ready[u] >= 0 && atomicCAS(next, -1, ready[u]) == -1) ready[u] = -1;  // kept
+    }
+    __syncwarp();
     ring2_push_warp(q, true, ready);
   }
 }
@@ -982,6 +994,20 @@ __device__ __forceinline__ void release_w_forward(const Ring2& q, const SolveArg
     --count;
   }
   ring2_push_span(q, true, first, count);
+}
+
+// The same by the whole CTA, after a barrier: a panel near the root has more
+// than a hundred tiles, whose slots one thread would store one after another.
+__device__ __forceinline__ void release_w_forward_cta(const Ring2& q, const SolveArgs& a, int t, SolveShared& sh) {
+  const int first = a.pv.ns + a.st_first[t];
+  if (threadIdx.x == 0) {
+    sh.keep = !sh.hold && sh.next < 0;
+    if (sh.keep) sh.next = first;
+  }
+  __syncthreads();
+  const int keep = sh.keep;
+  ring2_push_range(q, true, first + keep, a.nst[t] - keep, &sh.base);
+  __syncthreads();  // keep is rewritten for the next one
 }
 
 // TC: the instantiation whose FP64 panel tiles may run as split products on
@@ -1013,7 +1039,7 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
         sh.next = -1;
       } else {
         int lo_ready;
-        sh.task = ring2_claim(q, pend, &lo_ready, a.ntask_done);
+        sh.task = ring2_claim(q, pend, &lo_ready, a.ntask_done, nullptr, true);
       }
       // While this CTA holds a claimed slot whose task is not yet pushed, it
       // takes no continuation: it comes back for that task after this one.
@@ -1043,9 +1069,10 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
       // release the others
       if (a.nst[s] > 0 && a.ftdep) {
         // deterministic order: a tile also waits for its predecessors into the same panels
+        fence_gpu();
         for (int i = threadIdx.x; i < a.nst[s]; i += blockDim.x) {
           const int tile = a.st_first[s] + i;
-          if (atom_add_acqrel(&a.ftdep[tile], -1) == 1) keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + tile);
+          if (count_down(&a.ftdep[tile])) keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + tile);
         }
       } else if (a.nst[s] > 0) {
         const int keep = sh.hold ? 0 : 1;
@@ -1057,28 +1084,46 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
     } else if (task < ns + nst) {
       const int kt = task - ns, s = a.st_sn[kt];
       fwd_tile<T, FAN, TC>(a, s, kt - a.st_first[s], sm);
-      publish_cta_writes();
+      if (threadIdx.x == 0) {
+        sh.nw = 0;
+        sh.flag = 0;
+      }
+      __syncthreads();  // the tile's writes, for the signals of every thread
       // Counter updates are spread over the CTA's threads: a panel near the
-      // root has thousands of dependent tiles, and they sit on the critical path.
-      for (int e = a.st_tptr[kt] + threadIdx.x; e < a.st_tptr[kt + 1]; e += blockDim.x) {
+      // root has thousands of dependent tiles, and they sit on the critical
+      // path; the tile's own panel's count goes out beside them.
+      const int e0 = a.st_tptr[kt], e1 = a.st_tptr[kt + 1];
+      if (e0 + (int)threadIdx.x < e1 || threadIdx.x == blockDim.x - 1) fence_gpu();
+      for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
         const int t = a.st_tgt[e];
-        if (atom_add_acqrel(&a.fdep[t], -1) == 1) {
-          if (is_wpanel(a, t))
-            release_w_forward(q, a, t, sh.hold ? nullptr : &sh.next);
-          else
+        if (count_down(&a.fdep[t])) {
+          if (is_wpanel(a, t)) {
+            const int k = atomicAdd(&sh.nw, 1);
+            if (k < kWReady)
+              sh.wl[k] = t;
+            else
+              release_w_forward(q, a, t, nullptr);
+          } else {
             keep_or_push(q, sh.hold ? nullptr : &sh.next, t);
+          }
         }
       }
-      if (a.ftdep)  // deterministic order: the next tiles into the same panels
+      if (a.ftdep) {  // deterministic order: the next tiles into the same panels
+        fence_gpu();
         for (int e = a.ft_sptr[kt] + threadIdx.x; e < a.ft_sptr[kt + 1]; e += blockDim.x) {
           const int nx = a.ft_succ[e];
-          if (atom_add_acqrel(&a.ftdep[nx], -1) == 1) keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + nx);
+          if (count_down(&a.ftdep[nx])) keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + nx);
         }
-      if (threadIdx.x == 0) sh.flag = (atom_add_acqrel(&a.ftiles[s], -1) == 1);
+      }
+      if (threadIdx.x == blockDim.x - 1) sh.flag = count_down(&a.ftiles[s]);
       __syncthreads();
+      for (int k = 0; k < min(sh.nw, kWReady); ++k) release_w_forward_cta(q, a, sh.wl[k], sh);
       if (sh.flag) {
         if (is_wpanel(a, s)) {  // b_s is read by all: the diagonal task may overwrite it
-          if (threadIdx.x == 0) keep_or_push(q, sh.hold ? nullptr : &sh.next, s);
+          if (threadIdx.x == 0) {
+            fence_gpu();
+            keep_or_push(q, sh.hold ? nullptr : &sh.next, s);
+          }
         } else {
           release_tiles(q, nullptr, a.st_first[s], a.st_first[s] + a.nst[s], a.bdep, ns + nst,
                         sh.hold ? nullptr : &sh.next);
@@ -1090,17 +1135,17 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
       publish_cta_writes();
       // deterministic order: the panel's next backward tile
       if (a.ftdep && threadIdx.x == 0 && kt + 1 < a.st_first[s] + a.nst[s] &&
-          atom_add_acqrel(&a.bdep[kt + 1], -1) == 1)
+          count_down(&a.bdep[kt + 1]))
         keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + nst + kt + 1);
       if (is_wpanel(a, s)) {
         // the last backward tile completes x_s = y_s: it releases the tiles
         // that read it (the role of the backward diagonal task, which W panels
         // do not have)
-        if (threadIdx.x == 0) sh.flag = (atom_add_acqrel(&a.btiles[s], -1) == 1);
+        if (threadIdx.x == 0) sh.flag = count_down(&a.btiles[s]);
         __syncthreads();
         if (sh.flag)
           release_tiles(q, a.rt_tile, a.rt_ptr[s], a.rt_ptr[s + 1], a.bdep, ns + nst, sh.hold ? nullptr : &sh.next);
-      } else if (threadIdx.x == 0 && atom_add_acqrel(&a.btiles[s], -1) == 1) {
+      } else if (threadIdx.x == 0 && count_down(&a.btiles[s])) {
         keep_or_push(q, sh.hold ? nullptr : &sh.next, ns + 2 * nst + s);
       }
     } else {
@@ -1194,14 +1239,14 @@ __device__ void subtree_forward(const SolveArgs& a, int k, double* ys, double* z
     }
     // count the tiles down on the panels outside the subtree that they reach,
     // one (tile, target) entry per lane: the warp barrier orders every lane's
-    // writes before each lane's acq_rel decrement (and lane 0's fence)
+    // writes before each lane's fence
     if (__any_sync(0xffffffffu, outside)) {
-      if (lane == 0) __threadfence();
       __syncwarp();
+      fence_gpu();
       const int e0 = a.st_tptr[a.st_first[s]], e1 = a.st_tptr[a.st_first[s] + a.nst[s]];
       for (int e = e0 + lane; e < e1; e += 32) {
         const int t = a.st_tgt[e];
-        if (t > hi && atom_add_acqrel(&a.fdep[t], -1) == 1) {
+        if (t > hi && count_down(&a.fdep[t])) {
           if (is_wpanel(a, t))
             release_w_forward(q, a, t, nullptr);
           else
