@@ -158,7 +158,7 @@ typedef struct spchol_options {
                              x_s -= W^T x_below, with no diagonal solve between two steps of the
                              chain.  Costs the W buffer (the footprint counts it) and
                              2 (rows below) w^2 flops per such panel in the factorization.
-                             0 = default (32 for spchol_analyze, none for spchol_batch_analyze);
+                             0 = default (64 for spchol_analyze, none for spchol_batch_analyze);
                              -1 = none; not used with deterministic != 0 */
 } spchol_options;
 

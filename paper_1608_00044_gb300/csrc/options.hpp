@@ -12,7 +12,14 @@ namespace spchol {
 constexpr int kSolveTileRows = 64;  // rows per solve tile below the near-root band (staged in 32-row chunks)
 constexpr int kTrsmTileRows = 64;
 constexpr int kFp64TcMinWidth = 16;
-constexpr int kWDepth = 32;  // W panels (PlanParams::w_depth) of a single matrix, by default
+// W panels (PlanParams::w_depth) of a single matrix, by default.  Factorization
+// + solve, ms, by depth 32 / 64 / 96 / 128: 64^3 with 8 right-hand sides 383.0 +
+// 14.5 / 383.2 + 13.8 / 384.2 + 13.1 / 385.6 + 12.6, 27-point 48^3 with FP32
+// panels 12.48 + 7.55 / 12.53 + 6.88 / 13.00 + 6.59 / 13.06 + 6.55, 33 x 41 x
+// 37 with 16 17.8 + 4.49 / 18.0 + 3.95 / 18.2 + 3.83 / 18.1 + 3.83, 40^3 28.4 +
+// 3.94 / 28.6 + 3.51 / 29.0 + 3.29 / 28.9 + 3.27: 64 is the best of one
+// factorization and one solve.
+constexpr int kWDepth = 64;
 
 inline void default_options(spchol_options* o) {
   std::memset(o, 0, sizeof(*o));
