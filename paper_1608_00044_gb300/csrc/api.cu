@@ -62,6 +62,7 @@ struct spchol_handle_s {
   std::vector<int32_t> a_row, a_col;  // A's lower entries (original order); dropped after analyze
   int batch_count = 0;                // 0 = single matrix
   std::vector<int64_t> batch_n, batch_col0, batch_nnz0;  // per matrix: order, first column, first value
+  BatchItem* h_batch = nullptr;  // pinned: the running batch call's arrays, read by its kernels
   // device structures
   Arena arena;
   int32_t *d_fcol = nullptr, *d_nrows = nullptr, *d_ld = nullptr, *d_rows = nullptr, *d_parent = nullptr;
@@ -758,6 +759,23 @@ bool is_device_ptr(const void* p) {
     return false;
   }
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// Memory that a kernel of this handle may read as doubles.
+bool kernel_ptr(spchol_handle_t h, const void* p) {
+  cudaPointerAttributes at;
+  if (((uintptr_t)p & 7) != 0 || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (at.type == cudaMemoryTypeDevice && at.device == h->device) || at.type == cudaMemoryTypeManaged;
+}
+
+// The pinned table of a batch call's arrays.  The calls return after their
+// stream's work, so the next one may rewrite it.
+int batch_items(spchol_handle_t h) {
+  if (!h->h_batch) PINNED(h->h_batch, (size_t)h->batch_count * sizeof(BatchItem));
+  return 0;
 }
 
 int read_status(spchol_handle_t h, cudaStream_t st, int expect_done) {
@@ -1527,6 +1545,7 @@ int spchol_destroy(spchol_handle_t h) {
   pinned_put(h->h_prof, kProfWords * sizeof(unsigned long long));
   pinned_put(h->h_gmH, 3 * (kGmresRestart + 2) * sizeof(double));
   pinned_put(h->h_norms, h->h_norms_bytes);
+  pinned_put(h->h_batch, (size_t)h->batch_count * sizeof(BatchItem));
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);
   delete h;
@@ -1597,14 +1616,18 @@ int spchol_batch_factorize(spchol_handle_t h, const double* const* values, void*
   clear_stale_error();
   cudaStream_t st = (cudaStream_t)stream;
   const int cnt = h->batch_count;
+  int rc = batch_items(h);
+  if (rc) return rc;
   for (int i = 0; i < cnt; ++i) {
     const int64_t len = (i + 1 < cnt ? h->batch_nnz0[i + 1] : h->plan.nnz_a) - h->batch_nnz0[i];
-    if (len == 0) continue;
-    if (!values[i]) return -2;
-    const bool dev = is_device_ptr(values[i]);
-    CU(cudaMemcpyAsync(h->d_vals + h->batch_nnz0[i], values[i], len * sizeof(double),
-                       dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
+    if (len > 0 && !values[i]) return -2;
+    const bool by_kernel = len > 0 && kernel_ptr(h, values[i]);
+    h->h_batch[i] = BatchItem{const_cast<double*>(values[i]), h->batch_nnz0[i], by_kernel ? len : 0, 0, 0, 0};
+    if (len > 0 && !by_kernel)
+      CU(cudaMemcpyAsync(h->d_vals + h->batch_nnz0[i], values[i], len * sizeof(double),
+                         is_device_ptr(values[i]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
   }
+  CU(launch_batch_values(h->h_batch, cnt, h->d_vals, st));
   return factorize_impl(h, h->d_vals, nullptr, st);
 }
 
@@ -1626,17 +1649,27 @@ int spchol_batch_solve(spchol_handle_t h, double* const* B, const int64_t* ldb, 
   if (maxr == 0) return 0;
   const int64_t N = h->plan.n;
   int rc = ensure_workspace(h, N * maxr, maxr, st);
-  if (rc) return rc;
+  if (rc || (rc = batch_items(h))) return rc;
   // Gather every matrix's RHS into one N x maxr block (zero columns where a
-  // matrix has fewer right-hand sides), solve once, scatter back.
-  CU(cudaMemsetAsync(h->d_B, 0, N * maxr * sizeof(double), st));
+  // matrix has fewer right-hand sides), solve once, scatter back: device
+  // arrays by one kernel, host ones (and a device one that lies off an 8-byte
+  // boundary or on another device) by copies.
+  std::vector<int> copied;
   for (int i = 0; i < cnt; ++i) {
-    if (nrhs[i] == 0 || h->batch_n[i] == 0) continue;
+    const int64_t n = h->batch_n[i];
+    const bool any = nrhs[i] > 0 && n > 0;
+    const bool by_kernel = !any || kernel_ptr(h, B[i]);
+    h->h_batch[i] = BatchItem{B[i], h->batch_col0[i], by_kernel ? n : 0, ldb[i], nrhs[i], 0};
+    if (!by_kernel) copied.push_back(i);
+  }
+  if (!copied.empty()) CU(cudaMemsetAsync(h->d_B, 0, N * maxr * sizeof(double), st));
+  for (int i : copied) {
     const bool dev = is_device_ptr(B[i]);
     CU(cudaMemcpy2DAsync(h->d_B + h->batch_col0[i], N * sizeof(double), B[i], ldb[i] * sizeof(double),
                          h->batch_n[i] * sizeof(double), nrhs[i],
                          dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
   }
+  CU(launch_batch_rhs(h->h_batch, cnt, h->d_B, N, maxr, true, st));
   CU(cudaEventRecord(h->ev0, st));
   int core = 0;
   if (h->fp32) {
@@ -1649,8 +1682,8 @@ int spchol_batch_solve(spchol_handle_t h, double* const* B, const int64_t* ldb, 
     CU(launch_permute_out(h->d_Y, N, h->d_B, N, h->d_perm, N, maxr, st));
   }
   CU(cudaEventRecord(h->ev1, st));
-  for (int i = 0; i < cnt; ++i) {
-    if (nrhs[i] == 0 || h->batch_n[i] == 0) continue;
+  CU(launch_batch_rhs(h->h_batch, cnt, h->d_B, N, maxr, false, st));
+  for (int i : copied) {
     const bool dev = is_device_ptr(B[i]);
     CU(cudaMemcpy2DAsync(B[i], ldb[i] * sizeof(double), h->d_B + h->batch_col0[i], N * sizeof(double),
                          h->batch_n[i] * sizeof(double), nrhs[i],

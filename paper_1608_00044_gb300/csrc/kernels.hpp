@@ -200,6 +200,21 @@ constexpr size_t kNoallocScratchBytes = size_t(32) << 20;
 cudaError_t noalloc_scratch(int device, void** ptr);
 
 // mixed.cu
+// One matrix of a batch call, in pinned host memory that the kernels read:
+// the caller's device array (its values, or its right-hand sides with leading
+// dimension ld), and its first entry or column in the concatenated one.
+struct BatchItem {
+  double* p;
+  int64_t first, n, ld;
+  int32_t nrhs, pad;
+};
+// dst[first + e] = p[e], e < n, for every item (n = 0: none)
+cudaError_t launch_batch_values(const BatchItem* items, int count, double* dst, cudaStream_t st);
+// B (N rows, ld N, maxr columns) <-> the items' right-hand sides; the gather
+// writes zeros in the columns an item does not have
+cudaError_t launch_batch_rhs(const BatchItem* items, int count, double* B, int64_t N, int maxr, bool gather,
+                             cudaStream_t st);
+
 cudaError_t launch_residual(int64_t n, int nrhs, const int64_t* rp, const int32_t* ci, const int64_t* vmap,
                             const double* aval, const double* X, int64_t ldx, const double* B, int64_t ldb, double* R,
                             int64_t ldr, unsigned long long* colmax, cudaStream_t st);

@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 import threading
 
 import numpy as np
@@ -422,11 +423,12 @@ def destroy(h):
         h.value = None
 
 
-def _ptr_array(items, ctype=ctypes.c_void_p):
-    arr = (ctype * len(items))()
-    for i, x in enumerate(items):
-        arr[i] = _ptr(x) if ctype is ctypes.c_void_p else x
-    return arr
+def _ptr_array(items):
+    torch = sys.modules.get("torch")
+    tensor = torch.Tensor if torch is not None else ()
+    # a tensor's own checks first: a batch has hundreds of them
+    return (ctypes.c_void_p * len(items))(
+        *[x.data_ptr() if type(x) is tensor and x.is_contiguous() else _ptr(x) for x in items])
 
 
 def batch_analyze(ns, colptrs, rowinds, perms=None, opt: Options | None = None):
@@ -461,8 +463,8 @@ def batch_factorize(h, values, stream=None) -> int:
 def batch_solve(h, Bs, ldbs, nrhss, stream=None) -> int:
     count = len(Bs)
     arr = _ptr_array(list(Bs))
-    ld = (ctypes.c_int64 * count)(*[int(x) for x in ldbs])
-    nr = (ctypes.c_int * count)(*[int(x) for x in nrhss])
+    ld = (ctypes.c_int64 * count)(*map(int, ldbs))
+    nr = (ctypes.c_int * count)(*map(int, nrhss))
     rc = load().spchol_batch_solve(h, ctypes.addressof(arr), ctypes.addressof(ld), ctypes.addressof(nr),
                                    _stream(stream))
     if rc != 0:

@@ -871,3 +871,46 @@ def test_one_dense_panel_of_every_width(w, scale):
         bad[perm[w - 1], perm[w - 1]] *= -1.0
         assert s.factorize(lower(bad)) == 2
     s.close()
+
+
+@pytest.mark.parametrize("precision", ["FP64", "FP32"])
+def test_batch_arrays_on_host_and_device_off_alignment_and_of_different_shapes(precision):
+    # A batch call reads and writes device arrays by one kernel and the others
+    # by copies: matrices on the host, on the device and on the device off an
+    # 8-byte boundary, with no, one and several right-hand sides and padded
+    # leading dimensions, give the solutions of the batch that has all of them
+    # on the host (bitwise: deterministic mode), and the padding is left alone.
+    sides = [5, 17, 3, 30, 9, 12, 8]
+    nrhs = [1, 3, 0, 2, 1, 3, 2]
+    where = ["device", "host", "device", "device", "off", "off", "host"]
+    mats = [gridgen.diffusion_2d_5pt(s, sigma=1.0, seed=i) for i, s in enumerate(sides)]
+    o = spchol.default_options(precision=getattr(spchol, precision), deterministic=2)
+    h = spchol.batch_analyze([M.n for M in mats], [M.colptr for M in mats], [M.rowind for M in mats],
+                             [gridgen.geometric_nd(M.dims) for M in mats], o)
+    ld = [M.n + (i % 3) for i, M in enumerate(mats)]
+    rhs = [np.random.default_rng(i).uniform(-1.0, 1.0, (max(r, 1), l)) for i, (r, l) in enumerate(zip(nrhs, ld))]
+
+    def put(x, place):  # (the object whose address is passed, how to read it back)
+        if place == "host":
+            x = x.copy()
+            return x, x
+        raw = torch.zeros(x.nbytes + 16, dtype=torch.uint8, device="cuda")
+        at = 4 if place == "off" else 0
+        view = raw[at:at + x.nbytes]
+        view.copy_(torch.from_numpy(np.ascontiguousarray(x).reshape(-1).view(np.uint8)))
+        return view, view
+
+    back = lambda v, x: v if isinstance(v, np.ndarray) else v.cpu().numpy().view(np.float64).reshape(x.shape)
+    out = []
+    for places in (["host"] * len(mats), where):
+        vals = [put(M.values, p)[0] for M, p in zip(mats, places)]
+        assert spchol.batch_factorize(h, vals) == 0
+        X = [put(b, p)[0] for b, p in zip(rhs, places)]
+        spchol.batch_solve(h, X, ld, nrhs)
+        out.append([back(x, b) for x, b in zip(X, rhs)])
+    spchol.destroy(h)
+    for M, b, r, l, x0, x1 in zip(mats, rhs, nrhs, ld, *out):
+        assert np.array_equal(x0, x1)
+        assert np.array_equal(x1[:, M.n:], b[:, M.n:]) and (r > 0 or np.array_equal(x1, b))
+        if r > 0:
+            assert oracle.berr(M, np.asfortranarray(x1[:r, :M.n].T), np.asfortranarray(b[:r, :M.n].T)) <= 1e-12
