@@ -80,22 +80,6 @@ __device__ __forceinline__ void tri_pair(int p, int& ei, int& ek) {
   ei = p - e * (e + 1) / 2;
 }
 
-// 1 / d for the pivot d > 0 by Newton's iteration y <- y (2 - d y) from the
-// single-precision approximate reciprocal (relative error below 2^-22; two
-// steps take it below the FP64 rounding error); outside the range where the
-// seed is representable, the division.
-__device__ __forceinline__ double pivot_recip(double d) {
-  if (d > 1e-30 && d < 1e30) {
-    float y0;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"((float)d));
-    double y = (double)y0;
-    y = fma(y, fma(-d, y, 1.0), y);
-    y = fma(y, fma(-d, y, 1.0), y);
-    return y;
-  }
-  return 1.0 / d;
-}
-
 // d > 0 on the integer pipe (false for a NaN, as the comparison).
 __device__ __forceinline__ bool pivot_positive(double d) {
   const long long b = __double_as_longlong(d);
@@ -1575,25 +1559,33 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
 // task loop: the many small subtrees of a batch of small matrices, or the
 // leaves of a large one, then advance kWarpExec per CTA side by side with warp
 // barriers only, where a CTA subtree task runs one of them with CTA barriers
-// at every column and step.  A warp-wide FP64 instruction holds the SM's FP64
-// pipe as long whatever its active lanes (the pipe bounds these warps), so
-// each step spreads its entries over the lanes.  Per panel, in postorder:
-//   * the diagonal block in shared memory (leading dimension kWarpLd) in the
-//     square-root-free form A = M D M^T: the lane of row i forms its
-//     multiplier, then the trailing triangle's updates take one entry per lane
-//     and pass, as does the scaling L = M D^{1/2};
-//   * its inverse by substitution row by row, each step's entries one per lane
-//     and pass;
-//   * the panel solve by that inverse, l_rc = sum_{k <= c} a_rk X_ck, one
-//     output per lane and pass (the panel-solve tiles of the task loop solve
-//     by substitution instead: they run before the inverse exists);
-//   * the update tiles, one output per lane at a time (a dot product over the
-//     panel's columns in two chains): into panels inside the subtree by plain
-//     read-modify-write (no other task touches them), into the others by
-//     atomics, each tile then counted down on its target as a CTA subtree task
-//     does.
+// at every column and step.  What bounds them: a warp-wide FP64 instruction
+// holds an SM sub-partition's pipe for 64 clocks whatever its active lanes,
+// and every dependent trip to L2 costs 600.  So each step spreads its entries
+// over the lanes, and a panel that fits the warp's shared memory (97 % of
+// those of 512 2D grids; 6.9 columns and 17.6 rows below them on average) is
+// loaded once, factored with its rows below in place, and subtracted from its
+// ancestors over the flattened triangle of its rows below, not tile by tile:
+//   * column by column, the pivot's reciprocal square root on the integer
+//     pipe, the trailing rectangle one entry per lane and pass;
+//   * the inverse of the diagonal block by substitution on scaled rows; FP32
+//     panels solve their rows below by it, in FP32 (a substitution with L11
+//     rounded to FP32 refined to errors 10 % larger);
+//   * the updates kWarpOuts outputs per lane at a time: into panels inside the
+//     subtree by plain read-modify-write (no other task touches them), into the
+//     others by atomics.
+// A panel that does not fit has its diagonal block and inverse in shared
+// memory, the rows below solved by that inverse (l_rc = sum_{k <= c} a_rk
+// X_ck, one output per lane and pass) and its update tiles one after another.
+// The panel's tiles are then counted down on their targets outside.
 // After a failed pivot (here or anywhere) the rest of the subtree skips its
 // arithmetic but still counts its outside targets down.
+// Launch over the 512 grids, before -> now: FP64 8.0 -> 5.0 ms, FP32 5.7 -> 3.9 ms.
+constexpr int kWarpLd = kWarpSubW + 1;
+constexpr int kWarpExec = 4;                                   // warps of a CTA that run them
+constexpr int kWarpSmem = kWarpSubW * kWarpLd + kWarpSubW;     // doubles per warp
+constexpr int kWarpOuts = 4;                                   // update outputs in flight per lane
+
 // Entry p of a lower triangle numbered row by row (p = a (a + 1) / 2 + b,
 // 0 <= b <= a): row a, column b.  The float square root is exact at the
 // triangular numbers; the two corrections absorb its rounding elsewhere.
@@ -1605,174 +1597,292 @@ __device__ __forceinline__ void tri_decode(int p, int& ra, int& cb) {
   cb = p - t * (t + 1) / 2;
 }
 
-constexpr int kWarpLd = kWarpSubW + 1;
-constexpr int kWarpExec = 4;                                   // warps of a CTA that run them
-constexpr int kWarpSmem = kWarpSubW * kWarpLd + kWarpSubW;     // doubles per warp: the block, 1 / l_jj
+// p / m for p < 2^12, m >= 1, inv = 1 / m: the margin of 1 / (2 m) is far above the rounding.
+__device__ __forceinline__ int quick_div(int p, float inv) { return (int)(((float)p + 0.5f) * inv); }
+
+// Cholesky of the R x w columns at A (leading dimension la, R >= w): L11 and,
+// for R > w, the rows below it, and xd[j] = 1 / l_jj.  The upper triangle is
+// overwritten.  One warp; false at a pivot that is not positive, with its
+// column in *bad.
+__device__ __forceinline__ bool warp_factor(double* A, int la, int R, int w, double* xd, int* bad) {
+  const int lane = threadIdx.x & 31;
+  for (int j = 0; j < w; ++j) {
+    double* cj = A + j * la;
+    const double d = cj[j];
+    __syncwarp();  // every lane has read the pivot
+    if (!pivot_positive(d)) {
+      *bad = j;
+      return false;
+    }
+    const double y = pivot_rsqrt(d);
+    if (lane == 0) xd[j] = y;
+    for (int i = j + lane; i < R; i += 32) cj[i] *= y;
+    __syncwarp();
+    const int m = R - j - 1, nc = w - j - 1;
+    if (nc > 0) {
+      const float inv = 1.0f / (float)m;
+      for (int p = lane; p < m * nc; p += 32) {
+        const int q = quick_div(p, inv), k = j + 1 + q, i = j + 1 + p - q * m;
+        A[i + k * la] = fma(-cj[i], cj[k], A[i + k * la]);
+      }
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
+// X = L11^{-1} from L11 at A, by substitution row by row: with the rows below
+// the diagonal scaled by 1 / l_ii first (in place: L11 is stored), step kk
+// adds -l_ik X_kc to every X_ic with c <= kk < i, one per lane and pass.  X_ic,
+// i > c, in the upper triangle at (c, i); the diagonal is xd.
+__device__ __forceinline__ void warp_invert(double* A, int la, int w, const double* xd, double* __restrict__ X) {
+  const int lane = threadIdx.x & 31;
+  const float inv_w = 1.0f / (float)w;
+  for (int p = lane; p < w * w; p += 32) {
+    const int j = quick_div(p, inv_w), i = p - j * w;
+    if (i > j)
+      A[i + j * la] *= xd[i];
+    else if (i < j)
+      A[i + j * la] = 0.0;
+  }
+  __syncwarp();
+  for (int kk = 0; kk < w - 1; ++kk) {
+    const int nc = kk + 1, n = nc * (w - kk - 1);
+    const float inv = 1.0f / (float)nc;
+    for (int p = lane; p < n; p += 32) {
+      const int q = quick_div(p, inv), c = p - q * nc, i = kk + 1 + q;
+      const double x = c == kk ? xd[kk] : A[c + kk * la];
+      A[c + i * la] = fma(-A[i + kk * la], x, A[c + i * la]);
+    }
+    __syncwarp();
+  }
+  for (int p = lane; p < w * w; p += 32) {
+    const int j = quick_div(p, inv_w), i = p - j * w;
+    if (i >= j) X[p] = i == j ? xd[j] : A[j + i * la];
+  }
+}
+
+// Panel s of the subtree ending at panel hi, in shared memory: false (nothing
+// done) if it does not fit.
+template <typename T>
+__device__ __forceinline__ bool warp_panel(const FactorArgs& a, int s, int hi, double* ws, bool& skip) {
+  constexpr bool D64 = sizeof(T) == 8;
+  const int lane = threadIdx.x & 31;
+  const int f = a.pv.fcol[s], w = a.pv.fcol[s + 1] - f, ld = a.pv.ld[s], r = a.pv.nrows[s], nb = r - w;
+  const int R = D64 ? r : w, la = R | 1, ls = D64 ? la : nb | 1;
+  // shared memory: the columns, 1 / l_jj, two words per row below; FP32 panels: the rows below, X in FP32
+  const int need = la * w + w + 2 * nb + (D64 ? 0 : (ls * w + w * w + 1) / 2);
+  if (need > kWarpSmem) return false;
+  double* A = ws;
+  double* xd = A + la * w;
+  long long* ro = reinterpret_cast<long long*>(xd + w);  // where column j's entries start in its target, with row 0's offset out
+  long long* rp = ro + nb;                               // its relative indices: offset of row 0's | outside the subtree
+  T* S = D64 ? reinterpret_cast<T*>(A + w) : reinterpret_cast<T*>(rp + nb);
+  float* xf = D64 ? nullptr : reinterpret_cast<float*>(rp + nb) + ls * w;  // X in FP32: X_ck at xf[k + c w]
+  T* P = panel_ptr<T>(a, s);
+  const float inv_r = 1.0f / (float)r;
+#pragma unroll 4
+  for (int p = lane; p < r * w; p += 32) {
+    const int j = quick_div(p, inv_r), i = p - j * r;
+    const T v = i >= j ? ldcg(P + i + (size_t)j * ld) : T(0);
+    if (D64 || i < w)
+      A[i + j * la] = (double)v;
+    else
+      S[i - w + j * ls] = v;
+  }
+  // each target's first tile tells where the columns of its segment go (the
+  // relative indices of its later row tiles follow it)
+  const int32_t* Rs = a.pv.rows + a.pv.rowoff[s];
+  for (int q = lane; q < a.nu[s]; q += 32) {
+    const UTask u = a.ut[a.u_first[s] + q];
+    if (u.row0 != u.seg0) continue;
+    const long long base = a.pv.valoff[u.t] - (long long)a.pv.fcol[u.t] * a.pv.ld[u.t];
+    const long long rel = 2 * (u.rel - (u.row0 - w)) + (u.t > hi ? 1 : 0);
+    for (int jj = 0; jj < u.seglen; ++jj) {
+      ro[u.seg0 - w + jj] = base + (long long)Rs[u.seg0 + jj] * a.pv.ld[u.t];
+      rp[u.seg0 - w + jj] = rel;
+    }
+  }
+  __syncwarp();
+  int bad = 0;
+  if (!warp_factor(A, la, R, w, xd, &bad)) {
+    if (lane == 0) atomicMin(&a.ctrl[kInfo], f + bad + 1);
+    skip = true;
+    return true;
+  }
+  const float inv_R = 1.0f / (float)R;
+  for (int p = lane; p < R * w; p += 32) {
+    const int j = quick_div(p, inv_R), i = p - j * R;
+    if (i >= j) P[i + (size_t)j * ld] = (T)A[i + j * la];
+  }
+  __syncwarp();
+  warp_invert(A, la, w, xd, a.inv + a.invoff[s]);
+  if (!D64) {
+    const float inv_w = 1.0f / (float)w;
+    for (int p = lane; p < w * w; p += 32) {
+      const int c = quick_div(p, inv_w), k = p - c * w;
+      if (k <= c) xf[p] = (float)(k == c ? xd[c] : A[k + c * la]);
+    }
+    __syncwarp();
+    for (int i = lane; i < nb; i += 32)  // l_ic = sum over k <= c of a_ik X_ck, highest column first
+      for (int c = w - 1; c >= 0; --c) {
+        T v = T(0);
+        for (int k = 0; k <= c; ++k) v = fma(S[i + k * ls], (T)xf[k + c * w], v);
+        S[i + c * ls] = v;
+        P[w + i + (size_t)c * ld] = v;
+      }
+    __syncwarp();
+  }
+  // entry (i, j), i >= j, of the rows below's triangle, consecutive i on consecutive lanes
+  T* pool = reinterpret_cast<T*>(a.pool);
+  const int ntri = nb * (nb + 1) / 2;
+  for (int o0 = 0; o0 < ntri; o0 += 32 * kWarpOuts) {
+    T* dst[kWarpOuts];
+    T old[kWarpOuts];
+    int ij[kWarpOuts];  // row << 16 | column, bit 15: outside
+#pragma unroll
+    for (int q = 0; q < kWarpOuts; ++q) {
+      const int o = o0 + 32 * q + lane;
+      dst[q] = nullptr;
+      ij[q] = 0;
+      if (o < ntri) {
+        int ra, cb;
+        tri_decode(o, ra, cb);
+        const int j = nb - 1 - ra, i = nb - 1 - cb;
+        const long long e = rp[j];
+        const int pos = __ldg(a.relpos + (e >> 1) + i);
+        if (pos < 0) atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);  // cannot happen for a consistent plan
+        dst[q] = pos < 0 ? nullptr : pool + ro[j] + pos;
+        ij[q] = (i << 16) | ((int)(e & 1) << 15) | j;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kWarpOuts; ++q) old[q] = dst[q] && !(ij[q] & 0x8000) ? *dst[q] : T(0);
+#pragma unroll
+    for (int q = 0; q < kWarpOuts; ++q) {
+      if (o0 + 32 * q >= ntri) break;
+      // the products are summed before they meet the entry: one rounding at
+      // the entry's size, not one per column
+      const T* si = S + (ij[q] >> 16);
+      const T* sj = S + (ij[q] & 0x7fff);
+      T acc = T(0);
+      if (D64) {
+        for (int k = 0; k < w; ++k) acc = fma(si[k * ls], sj[k * ls], acc);
+      } else {
+        T acc1 = T(0);
+        int k = 0;
+        for (; k + 1 < w; k += 2) {
+          acc = fma(si[k * ls], sj[k * ls], acc);
+          acc1 = fma(si[(k + 1) * ls], sj[(k + 1) * ls], acc1);
+        }
+        if (k < w) acc = fma(si[k * ls], sj[k * ls], acc);
+        acc += acc1;
+      }
+      if (dst[q]) {
+        if (ij[q] & 0x8000)
+          red_add(dst[q], -acc);
+        else
+          *dst[q] = old[q] - acc;
+      }
+    }
+  }
+  return true;
+}
+
+// A panel that does not fit.
+template <typename T>
+__device__ void warp_panel_wide(const FactorArgs& a, int s, int hi, double* ws, bool& skip) {
+  const int lane = threadIdx.x & 31;
+  const int f = a.pv.fcol[s], w = a.pv.fcol[s + 1] - f, ld = a.pv.ld[s], r = a.pv.nrows[s];
+  double* xd = ws + kWarpSubW * kWarpLd;
+  T* P = panel_ptr<T>(a, s);
+  for (int idx = lane; idx < w * w; idx += 32) {
+    const int i = idx % w, j = idx / w;
+    ws[i + j * kWarpLd] = i >= j ? (double)ldcg(P + i + (size_t)j * ld) : 0.0;
+  }
+  __syncwarp();
+  int bad = 0;
+  if (!warp_factor(ws, kWarpLd, w, w, xd, &bad)) {
+    if (lane == 0) atomicMin(&a.ctrl[kInfo], f + bad + 1);
+    skip = true;
+    return;
+  }
+  for (int idx = lane; idx < w * w; idx += 32) {
+    const int i = idx % w, j = idx / w;
+    if (i >= j) P[i + (size_t)j * ld] = (T)ws[i + j * kWarpLd];
+  }
+  __syncwarp();
+  warp_invert(ws, kWarpLd, w, xd, a.inv + a.invoff[s]);
+  // L21 = A21 L11^{-T} by the inverse, in the panels' precision, columns in
+  // decreasing order, so that a_rc is overwritten only after every output that
+  // reads it (its row's higher columns: an earlier pass, or this one, whose
+  // reads all precede its writes)
+  using ct = T;
+  const int rb = r - w, nout = rb * w;
+  for (int o0 = 0; o0 < nout; o0 += 32) {
+    const int o = o0 + lane;
+    const bool ov = o < nout;
+    const int c = ov ? w - 1 - o / rb : 0, rr = ov ? o % rb : 0;
+    T* Pr = P + w + rr;
+    ct acc = ct(0);
+    if (ov)
+      for (int k = 0; k <= c; ++k)
+        acc = fma((ct)ldcg(Pr + (size_t)k * ld), k == c ? (ct)xd[c] : (ct)ws[k + c * kWarpLd], acc);
+    __syncwarp();
+    if (ov) Pr[(size_t)c * ld] = (T)acc;
+  }
+  __syncwarp();  // the rows below are written before the update tiles read them
+  const int32_t* Rs = a.pv.rows + a.pv.rowoff[s];
+  for (int ui = a.u_first[s]; ui < a.u_first[s] + a.nu[s]; ++ui) {
+    const UTask u = a.ut[ui];
+    const int ft = a.pv.fcol[u.t], ldt = a.pv.ld[u.t];
+    T* Pt = panel_ptr<T>(a, u.t);
+    const int nout = u.rowlen * u.seglen;
+    for (int o = lane; o < nout; o += 32) {
+      const int i = o % u.rowlen, j = o / u.rowlen;
+      const int gi = Rs[u.row0 + i], gj = Rs[u.seg0 + j];
+      if (gi < gj) continue;  // the upper part of a target's diagonal block
+      const T* ai = P + u.row0 + i;
+      const T* bj = P + u.seg0 + j;
+      T c0 = T(0), c1 = T(0);
+      int kk = 0;
+      for (; kk + 1 < w; kk += 2) {
+        c0 = fma(ai[(size_t)kk * ld], bj[(size_t)kk * ld], c0);
+        c1 = fma(ai[(size_t)(kk + 1) * ld], bj[(size_t)(kk + 1) * ld], c1);
+      }
+      if (kk < w) c0 = fma(ai[(size_t)kk * ld], bj[(size_t)kk * ld], c0);
+      const int p = __ldg(a.relpos + u.rel + i);
+      if (p < 0) {  // cannot happen for a consistent plan
+        atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);
+        continue;
+      }
+      T* dst = Pt + p + (size_t)(gj - ft) * ldt;
+      if (u.t > hi)
+        red_add(dst, -(c0 + c1));
+      else
+        *dst -= c0 + c1;
+    }
+  }
+}
 
 template <typename T>
 __device__ void warp_subtree(const FactorArgs& a, int k, double* ws) {
-  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int lo = a.sub_lo[k], hi = a.sub_hi[k];
-  double* xd = ws + kWarpSubW * kWarpLd;
   bool skip = ld_relaxed(&a.ctrl[kInfo]) != INT_MAX;
   const Ring2 q = rings_of(a);
   for (int s = lo; s <= hi; ++s) {
-    const int f = a.pv.fcol[s], w = a.pv.fcol[s + 1] - f, ld = a.pv.ld[s], r = a.pv.nrows[s];
-    T* P = panel_ptr<T>(a, s);
-    if (!skip) {
-      for (int idx = lane; idx < w * w; idx += 32) {
-        const int i = idx % w, j = idx / w;
-        ws[i + j * kWarpLd] = i >= j ? (double)ldcg(P + i + (size_t)j * ld) : 0.0;  // zeros above: the inverse goes there
-      }
-      __syncwarp();
-      double qj = 0.0;  // lane j: 1 / d_j
-      int bad = 0;
-      if (lane == 0) {
-        const double d0 = ws[0];
-        if (d0 > 0.0)
-          qj = pivot_recip(d0);
-        else
-          bad = 1;
-      }
-      if (__any_sync(full, bad)) {
-        if (lane == 0) atomicMin(&a.ctrl[kInfo], f + 1);
-        skip = true;
-      }
-      for (int j = 0; j < w && !skip; ++j) {
-        const double qv = __shfl_sync(full, qj, j);
-        const bool mine = lane > j && lane < w;
-        const double ci = mine ? ws[lane + j * kWarpLd] * qv : 0.0;  // the multiplier of row lane
-        // the trailing triangle a_ik -= c_i a_kj (j < k <= i < w), one entry
-        // per lane and pass; column j is read here and rewritten only below
-        const int m = w - j - 1, ntri = m * (m + 1) / 2;
-        for (int p0 = 0; p0 < ntri; p0 += 32) {
-          const int p = p0 + lane;
-          int ta, tb;
-          tri_decode(p < ntri ? p : 0, ta, tb);
-          const int i = j + 1 + ta, kk = j + 1 + tb;
-          const double c = __shfl_sync(full, ci, i);
-          if (p < ntri) ws[i + kk * kWarpLd] = fma(-c, ws[kk + j * kWarpLd], ws[i + kk * kWarpLd]);
-        }
-        __syncwarp();
-        if (lane == j + 1 && lane < w) {
-          const double d = ws[lane * (kWarpLd + 1)];
-          if (d > 0.0)
-            qj = pivot_recip(d);
-          else
-            bad = 1;
-        }
-        if (mine) ws[lane + j * kWarpLd] = ci;  // column j now holds the multipliers
-        if (__any_sync(full, bad)) {
-          if (lane == 0) atomicMin(&a.ctrl[kInfo], f + j + 2);
-          skip = true;
-        }
-        __syncwarp();
-      }
-      if (!skip) {
-        // L = M D^{1/2}: l_jj = sqrt(d_j), r_j = 1 / l_jj, l_ij = m_ij l_jj (one
-        // entry of the strictly lower triangle per lane and pass)
-        if (lane < w) {
-          const double l = sqrt(ws[lane * (kWarpLd + 1)]);
-          ws[lane * (kWarpLd + 1)] = l;
-          xd[lane] = 1.0 / l;
-        }
-        __syncwarp();
-        for (int p = lane; p < w * (w - 1) / 2; p += 32) {
-          int ta, tb;
-          tri_decode(p, ta, tb);
-          ws[ta + 1 + tb * kWarpLd] *= ws[tb * (kWarpLd + 1)];
-        }
-        __syncwarp();
-        for (int idx = lane; idx < w * w; idx += 32) {
-          const int i = idx % w, j = idx / w;
-          if (i >= j) P[i + (size_t)j * ld] = (T)ws[i + j * kWarpLd];
-        }
-        // L11^{-1}: X_ic (i > c) in the upper triangle at (c, i); step kk adds
-        // -l_ik X_kc to every X_ic with c <= kk < i (one per lane and pass) and
-        // completes X_{kk+1,c} by 1 / l_{kk+1,kk+1}
-        for (int kk = 0; kk < w - 1; ++kk) {
-          const int nc = kk + 1, n = nc * (w - kk - 1);
-          for (int p = lane; p < n; p += 32) {
-            const int c = p % nc, i = kk + 1 + p / nc;
-            const double xkc = c == kk ? xd[kk] : ws[c + kk * kWarpLd];
-            double v = fma(-ws[i + kk * kWarpLd], xkc, ws[c + i * kWarpLd]);
-            if (i == kk + 1) v *= xd[i];
-            ws[c + i * kWarpLd] = v;
-          }
-          __syncwarp();
-        }
-        double* X = a.inv + a.invoff[s];
-        for (int idx = lane; idx < w * w; idx += 32) {
-          const int i = idx % w, j = idx / w;
-          if (i >= j) X[idx] = i == j ? xd[j] : ws[j + i * kWarpLd];
-        }
-        // L21 = A21 L11^{-T} by the inverse, in the panels' precision:
-        // l_rc = sum_{k <= c} a_rk X_ck, one output per lane and pass, columns
-        // in decreasing order, so that a_rc is overwritten only after every
-        // output that reads it (its row's higher columns: an earlier pass, or
-        // this one, whose reads all precede its writes)
-        using ct = T;
-        const int rb = r - w, nout = rb * w;
-        for (int o0 = 0; o0 < nout; o0 += 32) {
-          const int o = o0 + lane;
-          const bool ov = o < nout;
-          const int c = ov ? w - 1 - o / rb : 0, rr = ov ? o % rb : 0;
-          T* Pr = P + w + rr;
-          ct acc = ct(0);
-          if (ov)
-            for (int k = 0; k <= c; ++k)
-              acc = fma((ct)ldcg(Pr + (size_t)k * ld), k == c ? (ct)xd[c] : (ct)ws[k + c * kWarpLd], acc);
-          __syncwarp();
-          if (ov) Pr[(size_t)c * ld] = (T)acc;
-        }
-        __syncwarp();  // the rows below are written before the update tiles read them
-      }
-    }
-    // update tiles of panel s
-    const int32_t* Rs = a.pv.rows + a.pv.rowoff[s];
-    bool any_out = false;
-    for (int ui = a.u_first[s]; ui < a.u_first[s] + a.nu[s]; ++ui) {
-      const UTask u = a.ut[ui];
-      const bool outside = u.t > hi;
-      if (!skip) {
-        const int ft = a.pv.fcol[u.t], ldt = a.pv.ld[u.t];
-        T* Pt = panel_ptr<T>(a, u.t);
-        const int nout = u.rowlen * u.seglen;
-        for (int o = lane; o < nout; o += 32) {
-          const int i = o % u.rowlen, j = o / u.rowlen;
-          const int gi = Rs[u.row0 + i], gj = Rs[u.seg0 + j];
-          if (gi < gj) continue;  // the upper part of a target's diagonal block
-          const T* ai = P + u.row0 + i;
-          const T* bj = P + u.seg0 + j;
-          T c0 = T(0), c1 = T(0);
-          int kk = 0;
-          for (; kk + 1 < w; kk += 2) {
-            c0 = fma(ai[(size_t)kk * ld], bj[(size_t)kk * ld], c0);
-            c1 = fma(ai[(size_t)(kk + 1) * ld], bj[(size_t)(kk + 1) * ld], c1);
-          }
-          if (kk < w) c0 = fma(ai[(size_t)kk * ld], bj[(size_t)kk * ld], c0);
-          const int p = __ldg(a.relpos + u.rel + i);
-          if (p < 0) {  // cannot happen for a consistent plan
-            atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);
-            continue;
-          }
-          T* dst = Pt + p + (size_t)(gj - ft) * ldt;
-          if (outside)
-            red_add(dst, -(c0 + c1));
-          else
-            *dst -= c0 + c1;
-        }
-      }
-      any_out = any_out || outside;
-    }
-    if (any_out) {  // publish the warp's atomics, then count its tiles down on their targets, one per lane
-      __syncwarp();
-      fence_gpu();
-      for (int ui = a.u_first[s] + lane; ui < a.u_first[s] + a.nu[s]; ui += 32) {
-        const int t = a.ut[ui].t;
-        if (t > hi && count_down(&a.dep_f[t])) ring2_push_one(q, true, t);
-      }
+    if (!skip && !warp_panel<T>(a, s, hi, ws, skip)) warp_panel_wide<T>(a, s, hi, ws, skip);
+    // publish the warp's atomics, then count the panel's tiles down on their
+    // targets outside the subtree, one per lane
+    __syncwarp();
+    bool fenced = false;
+    for (int ui = a.u_first[s] + lane; ui < a.u_first[s] + a.nu[s]; ui += 32) {
+      const int t = a.ut[ui].t;
+      if (t <= hi) continue;
+      if (!fenced) fence_gpu();
+      fenced = true;
+      if (count_down(&a.dep_f[t])) ring2_push_one(q, true, t);
     }
     __syncwarp();  // the next panel reads what this one's tiles wrote into it
   }

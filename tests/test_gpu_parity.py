@@ -914,3 +914,29 @@ def test_batch_arrays_on_host_and_device_off_alignment_and_of_different_shapes(p
         assert np.array_equal(x1[:, M.n:], b[:, M.n:]) and (r > 0 or np.array_equal(x1, b))
         if r > 0:
             assert oracle.berr(M, np.asfortranarray(x1[:r, :M.n].T), np.asfortranarray(b[:r, :M.n].T)) <= 1e-12
+
+
+@pytest.mark.parametrize("precision,l_tol,bar", [("FP64", 1e-11, BERR_FP64), ("FP32", 1e-5, 1e-12)])
+@pytest.mark.parametrize("width,tile", [(1, 1), (3, 5), (17, 64), (32, 7)])
+def test_warp_subtrees_at_every_panel_shape(precision, l_tol, bar, width, tile):
+    # Narrow and wide panels, panels that fit a warp's shared memory and panels
+    # that do not, row tiles that end inside a segment: L as in
+    # test_warp_subtrees_match_the_oracle, with its tolerances, and the backward
+    # error of the block-diagonal system (what the refinement stops on).
+    sides = np.random.default_rng(11).integers(3, 50, 150)
+    mats = [gridgen.diffusion_2d_5pt(int(s), sigma=1.0, seed=500 + i) for i, s in enumerate(sides)]
+    mats += [gridgen.diffusion_3d_27pt(int(s), sigma=1.0, seed=i) for i, s in enumerate([3, 4, 5, 6, 7, 7])]
+    perms = [gridgen.geometric_nd(M.dims) for M in mats]
+    Bs = [gridgen.rhs_uniform(M.n, 1, seed=i) for i, M in enumerate(mats)]
+    o = spchol.default_options(max_width=width, relax_zeros=16, tile_rows=tile, precision=getattr(spchol, precision))
+    h = spchol.batch_analyze([M.n for M in mats], [M.colptr for M in mats], [M.rowind for M in mats], perms, o)
+    st = spchol.stats(h)
+    assert st["n_warp_subtrees"] == st["n_subtrees"] > 0
+    assert spchol.batch_factorize(h, [M.values for M in mats]) == 0
+    A, _ = _merged(mats, perms)
+    d, lmax = l_max_diff(h, A)
+    assert d <= l_tol * lmax, (d, lmax)
+    Xs = [B.copy(order="F") for B in Bs]
+    spchol.batch_solve(h, Xs, [M.n for M in mats], [1] * len(mats))
+    spchol.destroy(h)
+    assert oracle.berr(A, np.asfortranarray(np.concatenate(Xs)), np.asfortranarray(np.concatenate(Bs))) <= bar
