@@ -68,6 +68,20 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// FP32 to FP64 on the integer pipe: a conversion instruction takes the FP64
+// pipe as long as two multiply-adds (119 clocks per warp and sub-partition;
+// this 34).  Normal numbers and zeros; the rest by the conversion.  For the
+// solves, whose every product with an FP32 panel needs one: 27-point 48^3, two
+// solves 6.9 -> 6.3 ms, 35 x 31 x 38 3.5 -> 2.9 ms.  (In the factorization,
+// where a block is widened once, beside other work, it was 2 % slower.)
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), u = b & 0x7fffffffu;
+  if (u - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((u >> 3) + 0x38000000u)), (int)(b << 29));
+  return u == 0 ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Loads of data that other CTAs of the same launch may have written: served
 // from L2, never from a possibly stale L1 line.
 __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }

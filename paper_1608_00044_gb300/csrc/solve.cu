@@ -719,12 +719,12 @@ __device__ void fwd_tile_fma(const SolveArgs& a, const T* P, int ld, int row0, i
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
         int k = k0;
         for (; k + 3 < k1; k += 4) {
-          s0 += (double)L[k * kTileLD] * y[k];
-          s1 += (double)L[(k + 1) * kTileLD] * y[k + 1];
-          s2 += (double)L[(k + 2) * kTileLD] * y[k + 2];
-          s3 += (double)L[(k + 3) * kTileLD] * y[k + 3];
+          s0 += widen(L[k * kTileLD]) * y[k];
+          s1 += widen(L[(k + 1) * kTileLD]) * y[k + 1];
+          s2 += widen(L[(k + 2) * kTileLD]) * y[k + 2];
+          s3 += widen(L[(k + 3) * kTileLD]) * y[k + 3];
         }
-        for (; k < k1; ++k) s0 += (double)L[k * kTileLD] * y[k];
+        for (; k < k1; ++k) s0 += widen(L[k * kTileLD]) * y[k];
         acc = (s0 + s1) + (s2 + s3);
       }
       if (parts > 1) {
@@ -895,12 +895,12 @@ __device__ void bwd_tile_fma(const SolveArgs& a, const T* P, int ld, int row0, i
           double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
           int i = ri0;
           for (; i + 3 < i1; i += 4) {
-            s0 += (double)lj[i] * xg[i];
-            s1 += (double)lj[i + 1] * xg[i + 1];
-            s2 += (double)lj[i + 2] * xg[i + 2];
-            s3 += (double)lj[i + 3] * xg[i + 3];
+            s0 += widen(lj[i]) * xg[i];
+            s1 += widen(lj[i + 1]) * xg[i + 1];
+            s2 += widen(lj[i + 2]) * xg[i + 2];
+            s3 += widen(lj[i + 3]) * xg[i + 3];
           }
-          for (; i < i1; ++i) s0 += (double)lj[i] * xg[i];
+          for (; i < i1; ++i) s0 += widen(lj[i]) * xg[i];
           part[q] += (s0 + s1) + (s2 + s3);
         }
       }
@@ -1221,10 +1221,10 @@ __device__ void subtree_forward(const SolveArgs& a, int k, double* ys, double* z
           double acc0 = 0.0, acc1 = 0.0;
           int kk = 0;
           for (; kk + 1 < w; kk += 2) {
-            acc0 = fma((double)Li[(size_t)kk * ld], zs[kk + c * w], acc0);
-            acc1 = fma((double)Li[(size_t)(kk + 1) * ld], zs[kk + 1 + c * w], acc1);
+            acc0 = fma(widen(Li[(size_t)kk * ld]), zs[kk + c * w], acc0);
+            acc1 = fma(widen(Li[(size_t)(kk + 1) * ld]), zs[kk + 1 + c * w], acc1);
           }
-          if (kk < w) acc0 = fma((double)Li[(size_t)kk * ld], zs[kk + c * w], acc0);
+          if (kk < w) acc0 = fma(widen(Li[(size_t)kk * ld]), zs[kk + c * w], acc0);
           const int g = R[row0 + i];
           double* dst = Y + g + (size_t)c * a.ldy;
           if (g < gend) {
@@ -1281,10 +1281,10 @@ __device__ void subtree_backward(const SolveArgs& a, int k, double* ys) {
           double acc0 = 0.0, acc1 = 0.0;
           int i = 0;
           for (; i + 1 < cnt; i += 2) {
-            acc0 = fma((double)Lj[i], ldcg(Y + R[row0 + i] + (size_t)c * a.ldy), acc0);
-            acc1 = fma((double)Lj[i + 1], ldcg(Y + R[row0 + i + 1] + (size_t)c * a.ldy), acc1);
+            acc0 = fma(widen(Lj[i]), ldcg(Y + R[row0 + i] + (size_t)c * a.ldy), acc0);
+            acc1 = fma(widen(Lj[i + 1]), ldcg(Y + R[row0 + i + 1] + (size_t)c * a.ldy), acc1);
           }
-          if (i < cnt) acc0 = fma((double)Lj[i], ldcg(Y + R[row0 + i] + (size_t)c * a.ldy), acc0);
+          if (i < cnt) acc0 = fma(widen(Lj[i]), ldcg(Y + R[row0 + i] + (size_t)c * a.ldy), acc0);
           ys[o] -= acc0 + acc1;
         }
       }

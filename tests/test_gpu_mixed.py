@@ -162,3 +162,23 @@ def test_tensor_core_ragged_widths(W):
     assert _l_rel_diff(h, A) <= 1e-5
     assert oracle.berr(A, X, b) <= BERR_MIXED
     spchol.destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["FP32", "TF32X3"])
+@pytest.mark.parametrize("exponent", [-120, -63, 0, 63, 116])
+def test_fp32_panels_of_every_scale(precision, exponent):
+    # The solves widen the panels' FP32 entries on the integer pipe for
+    # normal numbers and by conversions otherwise: a scaled system (exactly, by
+    # a power of four, so that its factor is scaled by a power of two), whose
+    # entries of L and of its square reach FP32's subnormal range and its upper
+    # end, has the unscaled one's solution, scaled, to the refinement's target.
+    A, perm, b = gridgen.workload("diff3d_8")
+    scaled = gridgen.CscLower(A.n, A.colptr, A.rowind, A.values * 2.0 ** exponent)
+    X = {}
+    for name, M in (("plain", A), ("scaled", scaled)):
+        s = spchol.SparseCholesky(M.n, M.colptr, M.rowind, perm, precision=getattr(spchol, precision))
+        assert s.factorize(M.values) == 0
+        X[name] = s.solve(np.asfortranarray(b.copy()))
+        assert oracle.berr(M, X[name], b) <= 1e-12
+        s.close()
+    assert np.abs(X["scaled"] * 2.0 ** exponent - X["plain"]).max() <= 1e-8 * np.abs(X["plain"]).max()
