@@ -362,6 +362,16 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   if (ok) invert_l11(sm, xd, w, X);
 }
 
+// The same as a function of its own: inlined into the kernel of the BF16-split
+// tiles it makes the registers of their hot loops spill (64^3: 140.1 -> 131.8
+// ms; the other kernels are faster with it inlined, 64^3 FP64 383.5 against
+// 386.9 ms, 64^2 0.437 against 0.477).
+template <typename T, bool FAN>
+__device__ __noinline__ void task_potrf_apart(const FactorArgs& a, int s, double* sm, FactorShared& sh, bool skip,
+                                              bool release) {
+  task_potrf<T, FAN>(a, s, sm, sh, skip, release);
+}
+
 // ---------------------------------------------------------------- FP64 operand slicing
 // Error-free splitting of a row of L for the BF16 tensor cores (the splitting
 // step of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
@@ -1250,13 +1260,18 @@ __device__ void task_update_oz(const FactorArgs& a, const UTask u, unsigned char
     // the slices themselves.
     // 16-byte pieces by cp.async (L2 only): every piece of the tile is in
     // flight at once instead of one load's latency per piece
-    for (int idx = tid; idx < kSlices * u.rowlen * chunks; idx += blockDim.x) {
-      const int c = idx % chunks, pr = idx / chunks;
-      const int p = pr / u.rowlen, r = pr - p * u.rowlen;
-      const uint16_t* src = sl + ((size_t)p * nb + (u.row0 - ws + r)) * kpad + 8 * c;
-      unsigned char* dst = A0 + p * arow + (r >> 3) * sbo + (r & 7) * 16 + c * 128;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-    }
+    // (at most 8 pieces a row: thread = row * 8 + piece, no index divisions)
+    const int pc = tid & 7;
+    if (pc < chunks)
+      for (int r = tid >> 3; r < u.rowlen; r += kFactorThreads / 8) {
+        const uint16_t* src = sl + (size_t)(u.row0 - ws + r) * kpad + 8 * pc;
+        const uint32_t dst = smem_addr(A0) + (r >> 3) * sbo + (r & 7) * 16 + pc * 128;
+#pragma unroll
+        for (int p = 0; p < kSlices; ++p)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + p * arow),
+                       "l"(src + (size_t)p * nb * kpad)
+                       : "memory");
+      }
     cp_async_commit();
     for (int cb = 0; cb < u.seglen; cb += kOzN) {
       const int ncol = min(kOzN, u.seglen - cb);
@@ -1264,12 +1279,16 @@ __device__ void task_update_oz(const FactorArgs& a, const UTask u, unsigned char
         gcol[j] = fan ? u.seg0 + cb + j : Rs[u.seg0 + cb + j];
         eb[j] = ldcg(ex + u.seg0 + cb + j);
       }
-      for (int idx = tid; idx < kSlices * ncol * chunks; idx += blockDim.x) {
-        const int c = idx % chunks, pr = idx / chunks;
-        const int p = pr / ncol, r = pr - p * ncol;
-        const uint16_t* src = sl + ((size_t)p * nb + (u.seg0 + cb - ws + r)) * kpad + 8 * c;
-        unsigned char* dst = B0 + p * brow + (r >> 3) * sbo + (r & 7) * 16 + c * 128;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+      {
+        const int r = (tid >> 3) & (kOzN - 1);
+        if (pc < chunks && r < ncol) {
+          const uint16_t* src = sl + (size_t)(u.seg0 + cb - ws + r) * kpad + 8 * pc;
+          const uint32_t dst = smem_addr(B0) + (r >> 3) * sbo + (r & 7) * 16 + pc * 128;
+          for (int p = tid / (8 * kOzN); p < kSlices; p += kFactorThreads / (8 * kOzN))
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + p * brow),
+                         "l"(src + (size_t)p * nb * kpad)
+                         : "memory");
+        }
       }
       cp_async_commit();
       cp_async_wait<0>();  // this thread's A (first pass) and B pieces have landed
@@ -1305,46 +1324,39 @@ __device__ void task_update_oz(const FactorArgs& a, const UTask u, unsigned char
       tc.phase ^= 1u;
       if (!ok && tid == 0) atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_ETIMEOUT);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // Epilogue: warp w reads TMEM lanes 32*(w%4).. (lanes 0..15 of them hold
-      // tile rows 16*(w%4)..) and a column half; warps whose rows or columns
-      // are all unused skip (tcgen05.ld is warp-collective, so the condition
-      // is warp-uniform).
-      const int quad = warp & 3, half = warp >> 2;
-      const int row = 16 * quad + lane;
-      constexpr int kHalf = kOzN / 2;
-      if (16 * quad < u.rowlen) {
-        for (int c0 = half * kHalf; c0 < half * kHalf + kHalf && c0 < ncol; c0 += 8) {
-          uint32_t v[kSlices][8];
+      // Epilogue: warp w reads rows 16 (w % 4) .. + 15 (TMEM lanes 32 (w % 4) ..)
+      // and the w / 4-th half of the columns of every group, as 16 x 256-bit
+      // fragments: lane l holds rows l / 4 and l / 4 + 8 at columns 2 (l % 4) and
+      // the next, so that every lane has four outputs (reading a row per lane
+      // left half of them idle; with the copies' index divisions gone, 64^3 160.8
+      // -> 141.1 ms).  tcgen05.ld is warp-collective: the condition is
+      // warp-uniform.
+      const int quad = warp & 3, c0 = (warp >> 2) * (kOzN / 2);
+      if (16 * quad < u.rowlen && c0 < ncol) {
+        uint32_t v[kSlices][4];
 #pragma unroll
-          for (int d = 0; d < kSlices; ++d) {
-            const uint32_t taddr = tc.tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d * kOzN + c0);
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3]), "=r"(v[d][4]),
-                           "=r"(v[d][5]), "=r"(v[d][6]), "=r"(v[d][7])
-                         : "r"(taddr));
-          }
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (ok && lane < 16 && row < u.rowlen && pos[row] >= 0) {
+        for (int d = 0; d < kSlices; ++d)
+          asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+                       : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3])
+                       : "r"(tc.tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d * kOzN + c0)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int j = c0 + q;
-              if (j < ncol && grow[row] >= gcol[j]) {
-                // t = sum_d v_d 2^(8 (6 - d)), C = t 2^(e_i + e_j - 64).  The group
-                // sums are integers below 2^25 in magnitude; t (< 2^75) is formed
-                // as hi 2^32 + lo and kept to 2^12 units in one int64, a
-                // truncation of at most 2^(e_i + e_j - 52), below the rounding
-                // bound of an FP64 dot product of these rows.
-                long long hi = 0, lo = 0;
+        for (int q = 0; q < 4; ++q) {
+          const int row = 16 * quad + (lane >> 2) + 8 * (q >> 1), j = c0 + 2 * (lane & 3) + (q & 1);
+          if (!ok || row >= u.rowlen || j >= ncol || pos[row] < 0 || grow[row] < gcol[j]) continue;
+          // t = sum_d v_d 2^(8 (6 - d)), C = t 2^(e_i + e_j - 64).  The group
+          // sums are integers below 2^25 in magnitude; t (< 2^75) is formed
+          // as hi 2^32 + lo and kept to 2^12 units in one int64, a
+          // truncation of at most 2^(e_i + e_j - 52), below the rounding
+          // bound of an FP64 dot product of these rows.
+          long long hi = 0, lo = 0;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) hi = hi * 256 + __float2int_rn(__uint_as_float(v[d][q]));
+          for (int d = 0; d < 3; ++d) hi = hi * 256 + __float2int_rn(__uint_as_float(v[d][q]));
 #pragma unroll
-                for (int d = 3; d < kSlices; ++d) lo = lo * 256 + __float2int_rn(__uint_as_float(v[d][q]));
-                const long long t12 = hi * (1ll << 20) + (lo >> 12);  // floor((hi 2^32 + lo) / 2^12)
-                const double c = fixed64_to_double(t12, ea[row] + eb[j] - 52);
-                scatter_put(Pt + pos[row] + (size_t)(gcol[j] - ft) * ldt, -c, fan);
-              }
-            }
-          }
+          for (int d = 3; d < kSlices; ++d) lo = lo * 256 + __float2int_rn(__uint_as_float(v[d][q]));
+          const long long t12 = hi * (1ll << 20) + (lo >> 12);  // floor((hi 2^32 + lo) / 2^12)
+          const double c = fixed64_to_double(t12, ea[row] + eb[j] - 52);
+          scatter_put(Pt + pos[row] + (size_t)(gcol[j] - ft) * ldt, -c, fan);
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -2102,7 +2114,10 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       }
     } else if (kind == 0) {
       type = 0;
-      task_potrf<T, FAN>(a, s, smd, sh, skip, release);
+      if constexpr (MODE == 3)
+        task_potrf_apart<T, FAN>(a, s, smd, sh, skip, release);
+      else
+        task_potrf<T, FAN>(a, s, smd, sh, skip, release);
     } else if (kind == 1) {
       type = 1;
       task_trsm<T, MODE>(a, s, si, smd, sh, skip, release);
