@@ -81,6 +81,7 @@ struct spchol_handle_s {
   int n_wsub = 0, grid_wsub = 0;  // the factorization's warp subtrees (0: none)
   int n_wsub_solve = 0;            // the solves' (0: none)
   int solve_done = 0;  // SolveArgs::ntask_done
+  int fuse_w = 0, factor_done = 0;  // FactorArgs::fuse_w, ntask_done
   int32_t *d_st_first = nullptr, *d_nst = nullptr, *d_st_sn = nullptr, *d_st_rows = nullptr, *d_kid_ptr = nullptr, *d_kids = nullptr;
   int32_t *d_nkids_init = nullptr, *d_fkids = nullptr, *d_ftiles = nullptr, *d_btiles = nullptr;
   int32_t *d_st_tptr = nullptr, *d_st_tgt = nullptr, *d_rt_ptr = nullptr, *d_rt_tile = nullptr;
@@ -415,6 +416,14 @@ int setup_device(spchol_handle_t h) {
     const int32_t missing = ns + P.n_trsm + P.n_u + P.in_sub[ns - 1];
     fseeds.erase(std::find(fseeds.begin(), fseeds.end(), missing));
   }
+  // panels whose diagonal task solves the rows below it: CUDA-core tiles only
+  // (not in the fan-in mode, whose panel-solve tiles wait for their own gathers)
+  h->fuse_w = P.flops <= kFuseFlops && mma_mode_of(h->opt.precision) == 0 && !P.params.fanin ? kFuseWidth : 0;
+  h->factor_done = P.n_factor_tasks;
+  for (int s = 0; s < ns; ++s) {
+    const int w = P.fcol[s + 1] - P.fcol[s];
+    if (P.in_sub[s] < 0 && P.ntrsm[s] == 1 && w <= h->fuse_w && fuse_shape(w, P.nrows[s] - w)) h->factor_done -= 1;
+  }
   size_t o_fseeds = r32(fseeds.size()), o_wsub = r32(warp_sub || warp_solve ? P.wsub.size() : 0);
   size_t o_stf = r32(ns), o_nst = r32(ns), o_strows = r32(ns), o_stsn = r32(P.st_sn.size()), o_kp = r32(ns + 1), o_k = r32(P.kids.size());
   // the panels of the warp subtrees: solved by the subtree solve launches, so
@@ -685,7 +694,7 @@ int setup_device(spchol_handle_t h) {
   if (fan) h->smem_factor = std::max(h->smem_factor, fanin_smem_bytes(wmax, h->fp32, &h->fan_cap));
   h->smem_solve = solve_smem_bytes(wmax, h->opt.precision == SPCHOL_FP64_TC, fan);
   int bf = 0, bs = 0;
-  CU(factor_configure(h->fp32, mma_mode_of(h->opt.precision), fan, h->smem_factor, &bf));
+  CU(factor_configure(h->fp32, mma_mode_of(h->opt.precision), fan, h->fuse_w > 0, h->smem_factor, &bf));
   if (h->n_wsub > 0 || h->n_wsub_solve > 0) {
     int bw = 0;
     CU(warp_subtree_configure(h->fp32, &bw));
@@ -845,6 +854,8 @@ int enqueue_factor(spchol_handle_t h, const double* vals, cudaStream_t st, bool 
   a.n_trsm = P.n_trsm;
   a.n_u = P.n_u;
   a.ntask = P.n_factor_tasks;
+  a.ntask_done = h->factor_done;
+  a.fuse_w = h->fuse_w;
   a.trsm_rows = P.params.trsm_rows;
   a.mma_mode = mma_mode_of(h->opt.precision);
   a.slices = h->d_slices;
@@ -897,7 +908,7 @@ int status_of(spchol_handle_t h) {
   const int* c = h->h_ctrl;
   if (c[kErr] != 0) return c[kErr];
   if (c[kInfo] != INT_MAX) return c[kInfo];
-  if (c[kDone] != h->plan.n_factor_tasks) return SPCHOL_EINTERNAL;
+  if (c[kDone] != h->factor_done) return SPCHOL_EINTERNAL;
   return 0;
 }
 

@@ -43,6 +43,13 @@ __device__ __forceinline__ Ring2 rings_of(const FactorArgs& a) {
   return Ring2{a.ring, a.ring + a.n_hi, a.n_hi, a.ntask - a.n_hi, a.ctrl, a.budget_ns};
 }
 
+// Panel s (w columns) has its rows below solved by its diagonal task (see
+// kFuseWidth).
+__device__ __forceinline__ bool fused_panel(const FactorArgs& a, int s, int w) {
+  const int nb = a.pv.nrows[s] - w;
+  return w <= a.fuse_w && a.ntrsm[s] == 1 && nb <= kFuseRows && w * w * nb <= kFuseWork;
+}
+
 template <typename T>
 __device__ __forceinline__ T* panel_ptr(const FactorArgs& a, int s) {
   return reinterpret_cast<T*>(a.pool) + a.pv.valoff[s];
@@ -296,7 +303,131 @@ __device__ void invert_l11(double* sm, const double* xd, int w, double* __restri
   }
 }
 
-template <typename T, bool FAN>
+// L21 = A21 L11^{-T} for rows row0 .. row0 + cnt - 1 of a panel at most
+// kTrsmMaxW wide, row by row: forward substitution along each row with the
+// columns in registers.  Warp q takes 4-row strips 4 (q + 8 v); lane (lr, lc)
+// holds row lr of the strip at columns lc + 8 cc.  Step c: the lane holding
+// column c scales it by rinv[c] = 1 / l_cc, the value is broadcast within the 8
+// lanes of the row, and every later column subtracts it times l_qc = Ls[q + ldl
+// c] (read past row w only for columns that are not stored).
+template <typename T>
+__device__ __forceinline__ void trsm_strips(T* P, int ld, int row0, int cnt, int w, const T* Ls, int ldl,
+                                            const T* rinv) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane >> 3, lc = lane & 7;
+  const int nstrip = (cnt + 3) >> 2;
+  for (int st = warp; st < nstrip; st += kFactorThreads / 32) {
+    const int rloc = 4 * st + lr;
+    const bool rv = rloc < cnt;
+    T* Pi = P + row0 + rloc;
+    T x[8];
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+      const int c = lc + 8 * cc;
+      x[cc] = (rv && c < w) ? ldcg(Pi + (size_t)c * ld) : T(0);
+    }
+#pragma unroll
+    for (int cbk = 0; cbk < 8; ++cbk) {
+      if (8 * cbk >= w) break;
+      for (int c8 = 0; c8 < 8; ++c8) {
+        const int c = 8 * cbk + c8;
+        if (c >= w) break;
+        if (lc == c8) x[cbk] *= rinv[c];
+        const T xc = __shfl_sync(0xffffffffu, x[cbk], (lr << 3) | c8);
+        const T* Lc = Ls + ldl * c;
+        if (lc > c8) x[cbk] -= xc * Lc[lc + 8 * cbk];
+#pragma unroll
+        for (int cc = cbk + 1; cc < 8; ++cc) {
+          if (8 * cc >= w) break;
+          x[cc] -= xc * Lc[lc + 8 * cc];
+        }
+      }
+    }
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+      const int c = lc + 8 * cc;
+      if (rv && c < w) Pi[(size_t)c * ld] = x[cc];
+    }
+  }
+}
+
+// Every row of panel s below its diagonal block is solved (published, and
+// acquired by thread 0 before a barrier): its update tiles are ready.  Whole
+// CTA.
+__device__ __forceinline__ void release_updates(const FactorArgs& a, int s, FactorShared& sh) {
+  const Ring2 q = rings_of(a);
+  const int first = a.pv.ns + a.n_trsm + a.u_first[s], nhi = a.nu_hi[s];
+  if (a.u_dep) {  // deterministic order: a tile also waits for its predecessor into the same target
+    fence_gpu();
+    for (int i = threadIdx.x; i < a.nu[s]; i += blockDim.x)
+      if (count_down(&a.u_dep[a.u_first[s] + i])) ring2_push_one(q, i < nhi, first + i);
+  } else {
+    ring2_push_range(q, true, first, nhi, &sh.base);
+    ring2_push_range(q, false, first + nhi, a.nu[s] - nhi, &sh.base);
+  }
+}
+
+// W = L21 L11^{-1} for rows row0 .. row0 + cnt - 1 of a W panel (Plan::woff):
+// each row w solves w L11 = l21 by back substitution, w_c = (l21_c - sum over
+// q > c of w_q l_qc) / l_cc for c = w-1 .. 0, from the rows this panel-solve
+// tile has just written and L11 (the inverse of the diagonal task is formed
+// after the release of these tiles, so it is not read here).  The layout of
+// the panel solve: warp q takes 4-row strips, lane (lr, lc) row lr at columns
+// lc + 8 cc; L11 is restaged with leading dimension 65, so that the 8 lanes of
+// a row read the entries l_c,lc+8cc of row c of L11 from distinct banks.
+template <typename T>
+__device__ void form_w_rows(const FactorArgs& a, int s, int row0, int cnt, double* smd) {
+  using ct = T;
+  constexpr int kLd = kTrsmMaxW + 1;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int w = a.pv.fcol[s + 1] - a.pv.fcol[s], ld = a.pv.ld[s];
+  const T* P = panel_ptr<T>(a, s);
+  T* W = reinterpret_cast<T*>(a.wbuf) + a.woff[s];
+  ct* Ls = reinterpret_cast<ct*>(smd);  // Ls[q + kLd c] = l_qc for q > c
+  ct* rinv = Ls + kLd * w;              // 1 / l_cc
+  __syncthreads();                      // the panel solve is done with shared memory
+  for (int idx = tid; idx < kTrsmMaxW * w; idx += nt) {
+    const int qq = idx & (kTrsmMaxW - 1), c = idx >> 6;
+    Ls[qq + kLd * c] = (qq < w && qq > c) ? (ct)ldcg(P + qq + (size_t)c * ld) : ct(0);
+  }
+  const double* Xd = a.inv + a.invoff[s];
+  for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));
+  __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31, lr = lane >> 3, lc = lane & 7;
+  const int nstrip = (cnt + 3) >> 2;
+  for (int st = warp; st < nstrip; st += nt >> 5) {
+    const int rloc = 4 * st + lr;
+    const bool rv = rloc < cnt;
+    const T* Pi = P + row0 + rloc;
+    ct x[8];
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+      const int c = lc + 8 * cc;
+      x[cc] = (rv && c < w) ? (ct)ldcg(Pi + (size_t)c * ld) : ct(0);
+    }
+#pragma unroll
+    for (int cbk = 7; cbk >= 0; --cbk) {
+      if (8 * cbk >= w) continue;
+      for (int c8 = 7; c8 >= 0; --c8) {
+        const int c = 8 * cbk + c8;
+        if (c >= w) continue;
+        if (lc == c8) x[cbk] *= rinv[c];
+        const ct xc = __shfl_sync(0xffffffffu, x[cbk], (lr << 3) | c8);
+        const ct* Lr = Ls + c;  // l_c,c' at Lr[kLd c'] for c' < c
+        if (lc < c8) x[cbk] -= xc * Lr[kLd * (lc + 8 * cbk)];
+#pragma unroll
+        for (int cc = 0; cc < cbk; ++cc) x[cc] -= xc * Lr[kLd * (lc + 8 * cc)];
+      }
+    }
+    T* Wi = W + row0 + rloc;
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+      const int c = lc + 8 * cc;
+      if (rv && c < w) Wi[(size_t)c * ld] = (T)x[cc];
+    }
+  }
+}
+
+template <typename T, bool FAN, bool FUSE>
 __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared& sh, bool skip, bool release = true) {
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
@@ -305,6 +436,7 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   double* xd = sm + w * w;  // 1 / l_jj, the diagonal of L11^{-1}
   double* X = a.inv + a.invoff[s];
   bool ok = true;
+  const bool fuse = FUSE && fused_panel(a, s, w);
   if (!skip) {
     stage_lower<true>(P, w, ld, sm);  // lower triangle; zeros above (used below for L11^{-1})
     const int uw = warp == 3 ? kUpdWarps - 1 : warp > 3 ? warp - 1 : warp;  // number among the update warps
@@ -343,6 +475,18 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
     }
     // a failed pivot, of this block or of any other: its columns are not used
     if (tid == 0) sh.flag = ld_relaxed(&a.ctrl[kInfo]) != INT_MAX;
+    if (FUSE && fuse) {  // the rows below, with L11 from shared memory (in the panel's type)
+      const int nb = a.pv.nrows[s] - w;
+      if constexpr (sizeof(T) == 8) {
+        trsm_strips<T>(P, ld, w, nb, w, sm, w, xd);
+      } else {
+        T *Lf = reinterpret_cast<T*>(xd + w), *rf = Lf + w * w;
+        for (int idx = tid; idx < w * w; idx += blockDim.x) Lf[idx] = (T)sm[idx];
+        for (int j = tid; j < w; j += blockDim.x) rf[j] = (T)xd[j];
+        __syncthreads();
+        trsm_strips<T>(P, ld, w, nb, w, Lf, w, rf);
+      }
+    }
     for (int j = warp; j < w; j += kFactorThreads / 32)
       for (int i = j + lane; i < w; i += 32) P[i + (size_t)j * ld] = (T)sm[i + j * w];
     // the panel-solve tiles scale by 1 / l_jj
@@ -357,9 +501,15 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
       if (count_down(&a.tdep[kt])) ring2_push_one(rings_of(a), true, a.pv.ns + kt);
     }
   } else if (release) {
-    ring2_push_range(rings_of(a), true, a.pv.ns + a.trsm_first[s], a.ntrsm[s], &sh.base);
+    if (FUSE && fuse)
+      release_updates(a, s, sh);
+    else
+      ring2_push_range(rings_of(a), true, a.pv.ns + a.trsm_first[s], a.ntrsm[s], &sh.base);
   }
-  if (ok) invert_l11(sm, xd, w, X);
+  if (ok) {
+    invert_l11(sm, xd, w, X);
+    if (FUSE && fuse && a.woff != nullptr && a.woff[s] >= 0) form_w_rows<T>(a, s, w, a.pv.nrows[s] - w, sm);
+  }
 }
 
 // The same as a function of its own: inlined into the kernel of the BF16-split
@@ -369,7 +519,7 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
 template <typename T, bool FAN>
 __device__ __noinline__ void task_potrf_apart(const FactorArgs& a, int s, double* sm, FactorShared& sh, bool skip,
                                               bool release) {
-  task_potrf<T, FAN>(a, s, sm, sh, skip, release);
+  task_potrf<T, FAN, false>(a, s, sm, sh, skip, release);
 }
 
 // ---------------------------------------------------------------- FP64 operand slicing
@@ -439,67 +589,6 @@ __device__ void slice_row(const double* Pi, int w, int ld, int kpad, int nb, int
 // ---------------------------------------------------------------- TRSM(s, k)
 // Arithmetic in the panel's type: FP64 panels solve in FP64, FP32 panels (the
 // mixed-precision modes) in FP32.
-// W = L21 L11^{-1} for rows row0 .. row0 + cnt - 1 of a W panel (Plan::woff):
-// each row w solves w L11 = l21 by back substitution, w_c = (l21_c - sum over
-// q > c of w_q l_qc) / l_cc for c = w-1 .. 0, from the rows this panel-solve
-// tile has just written and L11 (the inverse of the diagonal task is formed
-// after the release of these tiles, so it is not read here).  The layout of
-// the panel solve: warp q takes 4-row strips, lane (lr, lc) row lr at columns
-// lc + 8 cc; L11 is restaged with leading dimension 65, so that the 8 lanes of
-// a row read the entries l_c,lc+8cc of row c of L11 from distinct banks.
-template <typename T>
-__device__ void form_w_rows(const FactorArgs& a, int s, int row0, int cnt, double* smd) {
-  using ct = T;
-  constexpr int kLd = kTrsmMaxW + 1;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int w = a.pv.fcol[s + 1] - a.pv.fcol[s], ld = a.pv.ld[s];
-  const T* P = panel_ptr<T>(a, s);
-  T* W = reinterpret_cast<T*>(a.wbuf) + a.woff[s];
-  ct* Ls = reinterpret_cast<ct*>(smd);  // Ls[q + kLd c] = l_qc for q > c
-  ct* rinv = Ls + kLd * w;              // 1 / l_cc
-  __syncthreads();                      // the panel solve is done with shared memory
-  for (int idx = tid; idx < kTrsmMaxW * w; idx += nt) {
-    const int qq = idx & (kTrsmMaxW - 1), c = idx >> 6;
-    Ls[qq + kLd * c] = (qq < w && qq > c) ? (ct)ldcg(P + qq + (size_t)c * ld) : ct(0);
-  }
-  const double* Xd = a.inv + a.invoff[s];
-  for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, lr = lane >> 3, lc = lane & 7;
-  const int nstrip = (cnt + 3) >> 2;
-  for (int st = warp; st < nstrip; st += nt >> 5) {
-    const int rloc = 4 * st + lr;
-    const bool rv = rloc < cnt;
-    const T* Pi = P + row0 + rloc;
-    ct x[8];
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const int c = lc + 8 * cc;
-      x[cc] = (rv && c < w) ? (ct)ldcg(Pi + (size_t)c * ld) : ct(0);
-    }
-#pragma unroll
-    for (int cbk = 7; cbk >= 0; --cbk) {
-      if (8 * cbk >= w) continue;
-      for (int c8 = 7; c8 >= 0; --c8) {
-        const int c = 8 * cbk + c8;
-        if (c >= w) continue;
-        if (lc == c8) x[cbk] *= rinv[c];
-        const ct xc = __shfl_sync(0xffffffffu, x[cbk], (lr << 3) | c8);
-        const ct* Lr = Ls + c;  // l_c,c' at Lr[kLd c'] for c' < c
-        if (lc < c8) x[cbk] -= xc * Lr[kLd * (lc + 8 * cbk)];
-#pragma unroll
-        for (int cc = 0; cc < cbk; ++cc) x[cc] -= xc * Lr[kLd * (lc + 8 * cc)];
-      }
-    }
-    T* Wi = W + row0 + rloc;
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const int c = lc + 8 * cc;
-      if (rv && c < w) Wi[(size_t)c * ld] = (T)x[cc];
-    }
-  }
-}
-
 template <typename T, int MODE>
 __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, FactorShared& sh, bool skip,
                           bool release = true) {
@@ -513,12 +602,6 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
   ct* sm = reinterpret_cast<ct*>(smd);
   (void)f;
   if (!skip && w <= kTrsmMaxW) {
-    // L21 = A21 L11^{-T}, row by row: forward substitution along each row with
-    // the columns in registers.  Warp q takes 4-row strips 4 (q + 8 v); lane
-    // (lr, lc) holds row lr of the strip at columns lc + 8 cc.  Step c: the lane
-    // holding column c scales it by 1 / l_cc, the value is broadcast within the
-    // 8 lanes of the row, and every later column subtracts it times l_qc.
-    const int warp = tid >> 5, lane = tid & 31, lr = lane >> 3, lc = lane & 7;
     ct* Ls = sm;                        // Ls[q + 64 c] = l_qc for q > c, else 0
     ct* rinv = sm + kTrsmMaxW * w;      // 1 / l_cc
     for (int idx = tid; idx < kTrsmMaxW * w; idx += nt) {
@@ -528,40 +611,7 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
     const double* Xd = a.inv + a.invoff[s];
     for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));  // written by the diagonal task
     __syncthreads();
-    const int nstrip = (cnt + 3) >> 2;
-    for (int st = warp; st < nstrip; st += nt >> 5) {
-      const int rloc = 4 * st + lr;
-      const bool rv = rloc < cnt;
-      T* Pi = P + row0 + rloc;
-      ct x[8];
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        const int c = lc + 8 * cc;
-        x[cc] = (rv && c < w) ? (ct)ldcg(Pi + (size_t)c * ld) : ct(0);
-      }
-#pragma unroll
-      for (int cbk = 0; cbk < 8; ++cbk) {
-        if (8 * cbk >= w) break;
-        for (int c8 = 0; c8 < 8; ++c8) {
-          const int c = 8 * cbk + c8;
-          if (c >= w) break;
-          if (lc == c8) x[cbk] *= rinv[c];
-          const ct xc = __shfl_sync(0xffffffffu, x[cbk], (lr << 3) | c8);
-          const ct* Lc = Ls + kTrsmMaxW * c;
-          if (lc > c8) x[cbk] -= xc * Lc[lc + 8 * cbk];
-#pragma unroll
-          for (int cc = cbk + 1; cc < 8; ++cc) {
-            if (8 * cc >= w) break;
-            x[cc] -= xc * Lc[lc + 8 * cc];
-          }
-        }
-      }
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        const int c = lc + 8 * cc;
-        if (rv && c < w) Pi[(size_t)c * ld] = (T)x[cc];
-      }
-    }
+    trsm_strips<T>(P, ld, row0, cnt, w, Ls, kTrsmMaxW, rinv);
     if constexpr (sizeof(T) == 8 && MODE == 3) {
       if (w >= a.tc_min_width) {
         __syncthreads();  // the tile's rows are written (visible to this CTA through L2)
@@ -619,18 +669,7 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
   if (!release) return;  // inside a subtree task: no counters, the same CTA goes on
   if (tid == 0) sh.flag = count_down(&a.trsm_left[s]);
   __syncthreads();
-  if (sh.flag) {
-    const Ring2 q = rings_of(a);
-    const int first = a.pv.ns + a.n_trsm + a.u_first[s], nhi = a.nu_hi[s];
-    if (a.u_dep) {  // deterministic order: a tile also waits for its predecessor into the same target
-      fence_gpu();
-      for (int i = threadIdx.x; i < a.nu[s]; i += blockDim.x)
-        if (count_down(&a.u_dep[a.u_first[s] + i])) ring2_push_one(q, i < nhi, first + i);
-    } else {
-      ring2_push_range(q, true, first, nhi, &sh.base);
-      ring2_push_range(q, false, first + nhi, a.nu[s] - nhi, &sh.base);
-    }
-  }
+  if (sh.flag) release_updates(a, s, sh);
   // W rows after the release: the updates of this panel do not wait for them
   // (the solves, a later launch, read them)
   if (!skip && a.woff != nullptr && a.woff[s] >= 0) form_w_rows<T>(a, s, row0, cnt, smd);
@@ -1910,7 +1949,9 @@ __device__ void warp_subtree(const FactorArgs& a, int k, double* ws) {
 // their operand tiles' shared memory allows (a BF16-split CTA holds 128 of the
 // SM's 512 TMEM columns).  The fan-in mode's CUDA-core kernels run four: the
 // gather's staging area takes a quarter of the SM's shared memory.
-template <typename T, int MODE, bool FAN>
+// FUSE: the diagonal tasks of narrow panels solve the rows below them
+// (kFuseWidth).
+template <typename T, int MODE, bool FAN, bool FUSE>
 __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 : FAN ? 4 : sizeof(T) == 4 ? 6 : 5)
     factor_kernel(FactorArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1998,7 +2039,7 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
             ahead = -1;
           }
           int lo_ready;
-          sh.task = ring2_claim(q, pend, &lo_ready, a.ntask, &stash);
+          sh.task = ring2_claim(q, pend, &lo_ready, a.ntask_done, &stash);
           deep = lo_ready > 4 * (int)gridDim.x;
           if (sh.task >= 0 && pend[1] < 0 && pend[2] < 0 && stash < 0 && deep) ahead = atomicAdd(&q.ctrl[kHead], 2);
         }
@@ -2037,7 +2078,7 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
         sh.task = cur_task;
         int ph = cur_ph, i = cur_i + 1;
         if (ph == 0) {
-          ph = 1;
+          ph = FUSE && fused_panel(a, s, a.pv.fcol[s + 1] - a.pv.fcol[s]) ? 2 : 1;
           i = 0;
         }
         if (ph == 1 && i >= a.ntrsm[s]) {
@@ -2117,7 +2158,7 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       if constexpr (MODE == 3)
         task_potrf_apart<T, FAN>(a, s, smd, sh, skip, release);
       else
-        task_potrf<T, FAN>(a, s, smd, sh, skip, release);
+        task_potrf<T, FAN, FUSE>(a, s, smd, sh, skip, release);
     } else if (kind == 1) {
       type = 1;
       task_trsm<T, MODE>(a, s, si, smd, sh, skip, release);
@@ -2281,16 +2322,19 @@ size_t fanin_smem_bytes(int max_w, bool fp32, int* cap) {
 template <bool FAN>
 static const void* factor_fn_of(bool fp32, int mma_mode) {
   if (fp32)
-    return mma_mode == 0 ? (const void*)factor_kernel<float, 0, FAN> : (const void*)factor_kernel<float, 1, FAN>;
-  return mma_mode == 3 ? (const void*)factor_kernel<double, 3, FAN> : (const void*)factor_kernel<double, 0, FAN>;
+    return mma_mode == 0 ? (const void*)factor_kernel<float, 0, FAN, false>
+                         : (const void*)factor_kernel<float, 1, FAN, false>;
+  return mma_mode == 3 ? (const void*)factor_kernel<double, 3, FAN, false>
+                       : (const void*)factor_kernel<double, 0, FAN, false>;
 }
 
-static const void* factor_fn(bool fp32, int mma_mode, bool fan) {
+static const void* factor_fn(bool fp32, int mma_mode, bool fan, bool fuse) {
+  if (fuse) return fp32 ? (const void*)factor_kernel<float, 0, false, true> : (const void*)factor_kernel<double, 0, false, true>;
   return fan ? factor_fn_of<true>(fp32, mma_mode) : factor_fn_of<false>(fp32, mma_mode);
 }
 
-cudaError_t factor_configure(bool fp32, int mma_mode, bool fan, size_t smem, int* blocks_per_sm) {
-  const void* fn = factor_fn(fp32, mma_mode, fan);
+cudaError_t factor_configure(bool fp32, int mma_mode, bool fan, bool fuse, size_t smem, int* blocks_per_sm) {
+  const void* fn = factor_fn(fp32, mma_mode, fan, fuse);
   cudaError_t e = ensure_smem_limit(fn, smem);
   if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, kFactorThreads, smem);
@@ -2366,7 +2410,7 @@ cudaError_t launch_fanrec(const FanEnt* ent, int64_t n, const UTask* ut, const i
 
 cudaError_t launch_factor(bool fp32, const FactorArgs& a, int grid, size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<FactorArgs*>(&a)};
-  return cudaLaunchKernel(factor_fn(fp32, a.mma_mode, a.fan_ptr != nullptr), dim3(grid), dim3(kFactorThreads), args,
+  return cudaLaunchKernel(factor_fn(fp32, a.mma_mode, a.fan_ptr != nullptr, a.fuse_w > 0), dim3(grid), dim3(kFactorThreads), args,
                           smem, st);
 }
 

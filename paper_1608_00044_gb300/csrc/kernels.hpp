@@ -51,6 +51,8 @@ struct FactorArgs {
   const UTask* ut;
   const int32_t* relpos;  // relative row indices of the update tiles (UTask::rel)
   const unsigned char* tmaps;  // optional: one 128-byte TMA tensor map per panel (2-D view, see kUpdBox*)
+  int fuse_w;      // widest panel whose diagonal task solves its rows below (fuse_shape; 0: none)
+  int ntask_done;  // completed tasks at the end: ntask without the panel-solve tasks of those panels
   const int32_t* nu_hi;  // leading update tiles of each panel that go to the high-priority ring
   const int32_t* sub_lo;  // subtree tasks: first and last panel of each
   const int32_t* sub_hi;
@@ -176,7 +178,7 @@ cudaError_t launch_warp_subtrees(bool fp32, const FactorArgs& a, int grid, cudaS
 // Fan-in mode: shared memory a gather needs for panels up to max_w wide, and
 // the values it stages per batch (*cap).
 size_t fanin_smem_bytes(int max_w, bool fp32, int* cap);
-cudaError_t factor_configure(bool fp32, int mma_mode, bool fanin, size_t smem, int* blocks_per_sm);
+cudaError_t factor_configure(bool fp32, int mma_mode, bool fanin, bool fuse, size_t smem, int* blocks_per_sm);
 cudaError_t launch_assemble(bool fp32, const double* values, const int64_t* dest, int64_t nnz,
                             void* pool, cudaStream_t st);
 cudaError_t launch_factor(bool fp32, const FactorArgs& a, int grid, size_t smem, cudaStream_t st);

@@ -85,6 +85,21 @@ struct PlanParams {
 // Resident CTAs of the factorization the plan is laid out for: 152 SMs x 5.
 constexpr int kPlanCtas = 152 * 5;
 
+// In a small problem (at most kFuseFlops), a panel of at most kFuseWidth columns
+// with few rows below them (w^2 rows <= kFuseWork, at most kFuseRows) has a
+// single panel-solve tile, and its diagonal task solves those rows itself,
+// from the L11 it holds in shared memory: on the lower levels a task is mostly
+// its fixed costs (a claim, the panel's sizes, staging, publishing: 8 us of
+// the 8-column panel's 9), and the chain of a small problem is made of them.
+// Factorization before -> now, ms: 24^2 0.224 -> 0.178, 64^2 0.447 -> 0.415, 12^3
+// 0.840 -> 0.813, 27-point 20^3 2.29 -> 2.24, 181 x 203 1.59 -> 1.58, 250 x 256
+// 2.55 -> 2.50.  Larger ones are bound by their tiles, and the kernel that can
+// do it has more registers to spill (31 x 34 x 29 9.23 -> 9.34, 27-point 48^3
+// with FP32 panels 12.6 -> 13.1): they keep the kernel without it.
+constexpr int kFuseWidth = 32, kFuseRows = 64, kFuseWork = 32 * 32 * 32;
+constexpr double kFuseFlops = 1e9;
+inline bool fuse_shape(int w, int nb) { return w <= kFuseWidth && nb > 0 && nb <= kFuseRows && w * w * nb <= kFuseWork; }
+
 // Widest panel of a subtree task that runs on one warp (Plan::wsub).
 constexpr int kWarpSubW = 32;
 

@@ -415,6 +415,11 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
       solve_rows[d] = tr[nt[2 * d] >= prm.level_trsm * kPlanCtas ? 0 : nt[2 * d + 1] >= prm.level_trsm * kPlanCtas ? 1 : 2];
     }
   }
+  auto trsm_rows = [&](int32_t s) {
+    const int32_t w = P.fcol[s + 1] - P.fcol[s], nb = P.nrows[s] - w;
+    const bool one = P.flops <= kFuseFlops && fuse_shape(w, nb) && nb <= prm.trsm_rows;
+    return std::max(1, one ? std::max(nb, solve_rows[depth[s]]) : solve_rows[depth[s]]);
+  };
   auto update_rows = [&](int32_t s) {
     const bool tc = prm.tc_min_width > 0 && P.fcol[s + 1] - P.fcol[s] >= prm.tc_min_width;
     return std::max(1, tc ? prm.tc_tile_rows : upd_rows[depth[s]]);
@@ -425,7 +430,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     int64_t nt = 0, ntr = 0;
     for (int32_t s = 0; s < ns; ++s) {
       const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
-      const int TU = update_rows(s), TR = std::max(1, solve_rows[depth[s]]);
+      const int TU = update_rows(s), TR = trsm_rows(s);
       ntr += (r - w + TR - 1) / TR;
       const int32_t* R = P.rows.data() + P.rowoff[s];
       for (int32_t a = w; a < r;) {
@@ -443,7 +448,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
     const int32_t nb = r - w;
     const bool top = depth[s] < prm.top_depth;
-    const int TU = update_rows(s), TR = std::max(1, solve_rows[depth[s]]);
+    const int TU = update_rows(s), TR = trsm_rows(s);
     P.trsm_rows[s] = TR;
     P.trsm_first[s] = (int32_t)P.trsm_sn.size();
     P.ntrsm[s] = (nb + TR - 1) / TR;

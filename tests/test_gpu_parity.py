@@ -940,3 +940,21 @@ def test_warp_subtrees_at_every_panel_shape(precision, l_tol, bar, width, tile):
     spchol.batch_solve(h, Xs, [M.n for M in mats], [1] * len(mats))
     spchol.destroy(h)
     assert oracle.berr(A, np.asfortranarray(np.concatenate(Xs)), np.asfortranarray(np.concatenate(Bs))) <= bar
+
+
+@pytest.mark.parametrize("name,W", [("lap2d_24", 1), ("lap2d_24", 8), ("lap2d_33", 32), ("lap3d_8", 31), ("lap3d_9", 33),
+                                    ("diff3d_6", 64), ("diff3d_7", 24)])
+@pytest.mark.parametrize("precision,deterministic", [("FP64", 0), ("FP64", 1), ("FP32", 0)])
+def test_diagonal_tasks_that_solve_their_rows(name, W, precision, deterministic):
+    # Small problems: panels up to 32 wide solve the few rows below them in
+    # their diagonal task (with W of a near-root panel formed there too), wider
+    # ones and those with more rows do not.  L and the solution against the
+    # oracle's (1e-11 of max |L| in FP64, 1e-5 in FP32; berr 1e-13, refined 1e-12).
+    A, perm, b = gridgen.workload(name)
+    rc, X, st, h = gpu_factor_solve(A, perm, b, max_width=W, precision=getattr(spchol, precision),
+                                    deterministic=deterministic)
+    assert rc == 0
+    d, lmax = l_max_diff(h, A)
+    spchol.destroy(h)
+    assert d <= (1e-11 if precision == "FP64" else 1e-5) * lmax, (d, lmax)
+    assert oracle.berr(A, X, b) <= (BERR_FP64 if precision == "FP64" else 1e-12)
