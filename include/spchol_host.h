@@ -65,6 +65,10 @@ int spchol_plan_build(int64_t n, const int64_t* colptr, const int32_t* rowind, c
  */
 int spchol_plan_split_subtrees(spchol_plan_t p, int64_t max_steps);
 
+/* Split the fan-in gathers as the GPU library's analyze does (max_values < 0:
+ * at its own limit). */
+int spchol_plan_split_gathers(spchol_plan_t p, int64_t max_values);
+
 /* Length of array `what`, or -1 for an unknown id. */
 int64_t spchol_plan_len(spchol_plan_t p, int what);
 

@@ -92,15 +92,16 @@ struct spchol_handle_s {
   int32_t *d_ft_sptr = nullptr, *d_ft_succ = nullptr, *d_ft_dep0 = nullptr, *d_ftdep = nullptr;
   // fan-in mode (options.deterministic = 2): Plan::fan_* and the update
   // tiles' private buffers (a separate allocation, in the panels' type)
-  int64_t *d_fan_off = nullptr, *d_fan_ptr = nullptr;
+  int64_t* d_fan_off = nullptr;
   int32_t* d_fan_task = nullptr;
   FanEnt* d_fan_ent = nullptr;
+  GatherTask* d_gat = nullptr;
   FanRec* d_fan_rec = nullptr;  // the gather's records (a separate allocation)
   // fan-in solves: Plan::st_zf and friends, and the tiles' buffers for up to
   // fan_nrhs right-hand sides
   int64_t *d_st_zf = nullptr, *d_st_zb = nullptr;
   // fan-in gather tasks: Plan::gat_first and friends, and the live counters
-  int32_t *d_gat_first = nullptr, *d_gat_pc = nullptr, *d_pc_owner = nullptr, *d_gdiag0 = nullptr,
+  int32_t *d_gat_first = nullptr, *d_pc_owner = nullptr, *d_gdiag0 = nullptr,
           *d_tdep0 = nullptr, *d_gdiag = nullptr, *d_tdep = nullptr;
   Plan::SolveFanRec* d_rt_rec = nullptr;
   double *d_zf = nullptr, *d_zb = nullptr;
@@ -382,6 +383,7 @@ int setup_device(spchol_handle_t h) {
   // the others run on CTAs, none longer than a fair share of the launch (the
   // fault injection withholds the flop budget's task of the root)
   if (!warp_sub && h->opt.fault_inject == 0) split_subtrees(P, subtree_step_budget(P));
+  if (P.params.fanin && h->opt.fault_inject == 0) split_gathers(P, kGatherValues);
   Arena& A = h->arena;
   auto r32 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int32_t)); };
   auto r64 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int64_t)); };
@@ -461,11 +463,10 @@ int setup_device(spchol_handle_t h) {
          o_fdd = det ? r32(P.ft_dep0.size()) : 0;
   const bool fan = P.params.fanin;
   size_t o_fano = fan ? r64(P.fan_off.size()) : 0, o_fant = fan ? r32(P.fan_task.size()) : 0,
-         o_fanp = fan ? r64(P.fan_ptr.size()) : 0,
          o_fane = fan ? A.reserve(std::max<size_t>(P.fan_ent.size(), 1) * sizeof(FanEnt)) : 0,
          o_stzf = fan ? r64(P.st_zf.size()) : 0, o_stzb = fan ? r64(P.st_zb.size()) : 0,
          o_rtrec = fan ? A.reserve(std::max<size_t>(P.rt_rec.size(), 1) * sizeof(Plan::SolveFanRec)) : 0,
-         o_gatf = fan ? r32(P.gat_first.size()) : 0, o_gatp = fan ? r32(P.gat_pc.size()) : 0,
+         o_gatf = fan ? r32(P.gat_first.size()) : 0, o_gatp = fan ? A.reserve(std::max<size_t>(P.gat.size(), 1) * sizeof(GatherTask)) : 0,
          o_pco = fan ? r32(P.pc_owner.size()) : 0, o_gd0 = fan ? r32(P.gdiag0.size()) : 0,
          o_td0 = fan ? r32(P.tdep0.size()) : 0, o_gd = fan ? r32(P.gdiag0.size()) : 0,
          o_td = fan ? r32(P.tdep0.size()) : 0;
@@ -575,13 +576,12 @@ int setup_device(spchol_handle_t h) {
   if (fan) {
     h->d_fan_off = (int64_t*)(b + o_fano);
     h->d_fan_task = (int32_t*)(b + o_fant);
-    h->d_fan_ptr = (int64_t*)(b + o_fanp);
     h->d_fan_ent = (FanEnt*)(b + o_fane);
     h->d_st_zf = (int64_t*)(b + o_stzf);
     h->d_st_zb = (int64_t*)(b + o_stzb);
     h->d_rt_rec = (Plan::SolveFanRec*)(b + o_rtrec);
     h->d_gat_first = (int32_t*)(b + o_gatf);
-    h->d_gat_pc = (int32_t*)(b + o_gatp);
+    h->d_gat = (GatherTask*)(b + o_gatp);
     h->d_pc_owner = (int32_t*)(b + o_pco);
     h->d_gdiag0 = (int32_t*)(b + o_gd0);
     h->d_tdep0 = (int32_t*)(b + o_td0);
@@ -633,9 +633,9 @@ int setup_device(spchol_handle_t h) {
               (rc = upload(h, h->d_ft_dep0, P.ft_dep0))))
     return rc;
   if (fan && ((rc = upload(h, h->d_fan_off, P.fan_off)) || (rc = upload(h, h->d_fan_task, P.fan_task)) ||
-              (rc = upload(h, h->d_fan_ptr, P.fan_ptr)) || (rc = upload(h, h->d_fan_ent, P.fan_ent)) ||
+              (rc = upload(h, h->d_fan_ent, P.fan_ent)) ||
               (rc = upload(h, h->d_st_zf, P.st_zf)) || (rc = upload(h, h->d_st_zb, P.st_zb)) ||
-              (rc = upload(h, h->d_gat_first, P.gat_first)) || (rc = upload(h, h->d_gat_pc, P.gat_pc)) ||
+              (rc = upload(h, h->d_gat_first, P.gat_first)) || (rc = upload(h, h->d_gat, P.gat)) ||
               (rc = upload(h, h->d_pc_owner, P.pc_owner)) || (rc = upload(h, h->d_gdiag0, P.gdiag0)) ||
               (rc = upload(h, h->d_tdep0, P.tdep0)) || (rc = upload(h, h->d_rt_rec, P.rt_rec))))
     return rc;
@@ -873,14 +873,13 @@ int enqueue_factor(spchol_handle_t h, const double* vals, cudaStream_t st, bool 
     a.fan_buf = h->d_fan_buf;
     a.fan_off = h->d_fan_off;
     a.fan_task = h->d_fan_task;
-    a.fan_ptr = h->d_fan_ptr;
     a.fan_rec = h->d_fan_rec;
     CU(cudaMemcpyAsync(h->d_gdiag, h->d_gdiag0, (size_t)P.ns * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     if (P.n_trsm > 0)
       CU(cudaMemcpyAsync(h->d_tdep, h->d_tdep0, (size_t)P.n_trsm * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     a.gat0 = P.ns + P.n_trsm + P.n_u + P.n_sub;
     a.gat_first = h->d_gat_first;
-    a.gat_pc = h->d_gat_pc;
+    a.gat = h->d_gat;
     a.pc_owner = h->d_pc_owner;
     a.gdiag0 = h->d_gdiag0;
     a.gdiag = h->d_gdiag;

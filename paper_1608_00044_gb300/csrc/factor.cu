@@ -1410,7 +1410,8 @@ __device__ void task_update_oz(const FactorArgs& a, const UTask u, unsigned char
 // Deterministic fan-in mode (the fan-in family of Section II-C, restated for
 // one GPU): update tiles store their products in private buffers, and a
 // gather task per piece of a target panel's rows (at most kFanPieceRows rows,
-// all columns) adds them in, tile after tile in the piece's list order, before
+// all columns or, where the list is long, a window of them: split_gathers) adds
+// them in, tile after tile in the piece's list order, before
 // the task that owns those rows factors or solves them; every entry of L thus
 // receives its updates in one fixed order whatever the schedule, and the
 // pieces of one panel are gathered in parallel.  The piece sits in shared
@@ -1421,7 +1422,16 @@ __device__ void task_update_oz(const FactorArgs& a, const UTask u, unsigned char
 //      hold its rows in the piece (cp.async, L2 only: the buffers were written
 //      by other CTAs; every copy of the batch in flight at once) and load the
 //      rows' positions in the piece and the columns' positions in the panel;
-//   3. the values are added tile by tile (a barrier between tiles).
+//   3. the values are added tile by tile: with a barrier between tiles, or --
+//      for at most kFanOwn columns, which most split gathers and the narrow
+//      panels have -- each thread adding to the one entry it owns, in a
+//      register, from maps of where the tiles' rows and columns lie.
+// What bounds it: the latency of a tile's step (0.35 us with the barrier; a
+// tile has 107 values in a piece on average), one after another in the top
+// separators' pieces.  Factorization of a 27^3 Laplacian: 12.0 ms; split 8.8;
+// and with the threads' own entries 8.0.  (Columns dealt out to the warps
+// without barriers, whatever the width, was slower: 14.5 and split 9.9 -- each
+// warp's FP64 add holds the pipe for 64 clocks, however few lanes it has.)
 // The piece and the buffers are read around L1; the records were written at
 // analysis.
 struct FanMeta {
@@ -1434,6 +1444,10 @@ struct FanMeta {
 };
 constexpr int kFanBatch = 32;
 constexpr int kFanVcap = 1024;  // staged positions per batch (a tile has at most 32 + 128)
+constexpr int kFanOwn = kFactorThreads / 32;  // columns of a piece whose entries the threads own
+constexpr int kFanAhead = 4;                  // tiles whose values are read before the first is added
+static_assert(kFanPieceRows == 32 && kFanVcap * sizeof(int16_t) >= kFanBatch * (32 + 4 * kFanOwn),
+              "the owners' maps take the positions' place");
 constexpr size_t kFanMetaBytes = ((kFanBatch * sizeof(FanMeta) + 16) + 15) & ~size_t(15);
 
 // 16-byte pieces that can hold ni consecutive values starting anywhere.
@@ -1452,14 +1466,17 @@ __device__ __forceinline__ int fan_tile_of(const FanMeta* meta, int nb, int idx,
 }
 
 template <typename T>
-__device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np, unsigned char* smraw) {
+__device__ void fanin_gather(const FactorArgs& a, int t, const GatherTask& G, int p0, int np, unsigned char* smraw) {
   constexpr int E = 16 / (int)sizeof(T);  // values per 16-byte piece
   const int tid = threadIdx.x, nt = blockDim.x;
-  long long e = a.fan_ptr[pc];
-  const long long e1 = a.fan_ptr[pc + 1];
+  long long e = G.e0;
+  const long long e1 = G.e1;
   if (e == e1) return;  // nothing lands in these rows
-  const int ft = a.pv.fcol[t], wt = a.pv.fcol[t + 1] - ft, ldt = a.pv.ld[t];
-  T* Pt = panel_ptr<T>(a, t);
+  // its columns [G.c0, G.c1) of the panel: numbered from 0 here, and rows from
+  // position c on have entries in its column c
+  const int ft = a.pv.fcol[t] + G.c0, wt = G.c1 - G.c0, ldt = a.pv.ld[t];
+  const int d0 = p0 - G.c0;
+  T* Pt = panel_ptr<T>(a, t) + (size_t)G.c0 * ldt;
   const T* F = reinterpret_cast<const T*>(a.fan_buf);
   const int cap = a.fan_cap;  // 16-byte pieces per batch; one tile's always fit
   unsigned char* base = smraw + ((16u - (smem_addr(smraw) & 15u)) & 15u);
@@ -1468,9 +1485,20 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
   int16_t* pv = reinterpret_cast<int16_t*>(base + kFanMetaBytes);  // positions: rows in the piece, then columns
   T* Bs = reinterpret_cast<T*>(pv + kFanVcap);                     // the staged pieces
   T* S = Bs + (size_t)cap * E;  // the piece: np rows x wt columns, leading dimension kFanPieceRows
-  for (int idx = tid; idx < np * wt; idx += nt) {
-    const int p = idx % np, c = idx / np;
-    S[p + kFanPieceRows * c] = ldcg(Pt + p0 + p + (size_t)c * ldt);
+  // at most one column a warp: a thread owns the entry (lane, warp)
+  const int lane = tid & 31, warp = tid >> 5;
+  const bool own = wt <= kFanOwn;
+  T acc = T(0);
+  int8_t* rowof = reinterpret_cast<int8_t*>(pv);              // [kFanBatch][32]: the tile's row there, or -1
+  int32_t* colof = reinterpret_cast<int32_t*>(rowof + kFanBatch * 32);  // [kFanBatch][kFanOwn]: its column's
+                                                                        // first staged value, or -1
+  if (own) {
+    if (lane < np && warp < wt) acc = ldcg(Pt + p0 + lane + (size_t)warp * ldt);
+  } else {
+    for (int idx = tid; idx < np * wt; idx += nt) {
+      const int p = idx % np, c = idx / np;
+      S[p + kFanPieceRows * c] = ldcg(Pt + p0 + p + (size_t)c * ldt);
+    }
   }
   FanRec r{};  // warp 0: the records of the next batch window
   if (tid < 32 && e + tid < e1) r = a.fan_rec[e + tid];
@@ -1517,6 +1545,8 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
       }
       r = FanRec{};
       if (e + nb + tid < e1) r = a.fan_rec[e + nb + tid];  // in flight during this batch
+    } else if (own) {
+      for (int idx = tid - 32; idx < kFanBatch * (8 + kFanOwn); idx += nt - 32) reinterpret_cast<int32_t*>(rowof)[idx] = -1;
     }
     __syncthreads();
     if (prof) {
@@ -1546,7 +1576,8 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
     }
     cp_async_commit();
     for (int idx = tid; idx < npos; idx += nt) {
-      const FanMeta& mk = meta[fan_tile_of(meta, nb, idx, false)];
+      const int k = fan_tile_of(meta, nb, idx, false);
+      const FanMeta& mk = meta[k];
       const int lv = idx - mk.pre_v;
       int q;
       bool ok;
@@ -1558,7 +1589,16 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
         ok = q >= 0 && q < wt;
       }
       if (!ok) atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);  // outside the piece: an inconsistent plan
-      pv[idx] = ok ? (int16_t)q : (int16_t)-1;
+      if (!own) {
+        pv[idx] = ok ? (int16_t)q : (int16_t)-1;
+      } else if (ok) {
+        const int j = lv - mk.ni;
+        if (j < 0)
+          rowof[k * 32 + q] = (int8_t)lv;
+        else
+          colof[k * kFanOwn + q] =
+              (mk.pre_b + j * mk.cps) * E + (int)((mk.fo + (long long)j * mk.rowlen) & (E - 1));
+      }
     }
     cp_async_wait<0>();
     __syncthreads();
@@ -1568,7 +1608,26 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
       tq = tn;
     }
     // 3. tile by tile: an entry's updates land in list order
-    for (int k = 0; k < nb; ++k) {
+    if (own && warp < wt && d0 + np > warp) {  // (the warp's column has rows in the lower triangle)
+      for (int k0 = 0; k0 < nb; k0 += kFanAhead) {
+        int col[kFanAhead], row[kFanAhead];
+        T x[kFanAhead];
+#pragma unroll
+        for (int u = 0; u < kFanAhead; ++u) {
+          col[u] = k0 + u < nb ? colof[(k0 + u) * kFanOwn + warp] : -1;  // the same in every lane
+          row[u] = k0 + u < nb && d0 + lane >= warp ? rowof[(k0 + u) * 32 + lane] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kFanAhead; ++u) x[u] = col[u] >= 0 && row[u] >= 0 ? Bs[col[u] + row[u]] : T(0);
+#pragma unroll
+        for (int u = 0; u < kFanAhead; ++u)
+          if (col[u] >= 0) {
+            const T y = acc + x[u];
+            if (row[u] >= 0) acc = y;
+          }
+      }
+    }
+    for (int k = 0; !own && k < nb; ++k) {
       const FanMeta& mk = meta[k];
       const int ni = mk.ni, n = ni * mk.seglen;
       for (int idx = tid; idx < n; idx += nt) {
@@ -1576,7 +1635,7 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
         const int j = (int)(((float)idx + 0.5f) * mk.inv_ni), ii = idx - j * ni;
         const int p = pv[mk.pre_v + ii], c = pv[mk.pre_v + ni + j];
         // lower triangle of the target (rows below its diagonal block always are)
-        if (p >= 0 && c >= 0 && (p0 + p >= wt || p0 + p >= c)) {
+        if (p >= 0 && c >= 0 && d0 + p >= c) {
           const int sub = (int)((mk.fo + (long long)j * mk.rowlen) & (E - 1));
           S[p + kFanPieceRows * c] += Bs[(size_t)(mk.pre_b + j * mk.cps) * E + sub + ii];
         }
@@ -1592,9 +1651,13 @@ __device__ void fanin_gather(const FactorArgs& a, int t, int pc, int p0, int np,
     }
     e += nb;
   }
-  for (int idx = tid; idx < np * wt; idx += nt) {
-    const int p = idx % np, c = idx / np;
-    Pt[p0 + p + (size_t)c * ldt] = S[p + kFanPieceRows * c];
+  if (own) {
+    if (lane < np && warp < wt) Pt[p0 + lane + (size_t)warp * ldt] = acc;
+  } else {
+    for (int idx = tid; idx < np * wt; idx += nt) {
+      const int p = idx % np, c = idx / np;
+      Pt[p0 + p + (size_t)c * ldt] = S[p + kFanPieceRows * c];
+    }
   }
   if (prof) {
     for (int k = 0; k < 3; ++k) atomicAdd(&a.prof[10 + k], (unsigned long long)tp[k]);
@@ -2132,7 +2195,8 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
       // fan-in mode: a gather task adds the buffered updates of one row piece
       // of a panel, then counts down the task that owns those rows
       type = 0;
-      const int pc = a.gat_pc[si], o = a.pc_owner[pc];
+      const GatherTask G = a.gat[si];
+      const int pc = G.pc, o = a.pc_owner[pc];
       const int t = o < a.pv.ns ? o : a.trsm_sn[o - a.pv.ns];
       const int w = a.pv.fcol[t + 1] - a.pv.fcol[t];
       int p0, p1;
@@ -2144,7 +2208,7 @@ __global__ void __launch_bounds__(kFactorThreads, MODE == 3 ? 3 : MODE != 0 ? 2 
         p0 = r0 + (pc - a.fan_task[o]) * kFanPieceRows;
         p1 = min(min(a.pv.nrows[t], r0 + tr), p0 + kFanPieceRows);
       }
-      if (!skip) fanin_gather<T>(a, t, pc, p0, p1 - p0, smem_raw);
+      if (!skip) fanin_gather<T>(a, t, G, p0, p1 - p0, smem_raw);
       publish_cta_writes();
       if (threadIdx.x == 0) {
         if (o < a.pv.ns) {
@@ -2390,12 +2454,12 @@ __global__ void fanrec_kernel(const FanEnt* __restrict__ ent, int64_t n, const U
     const FanEnt fe = ent[k];
     const UTask u = ut[fe.u];
     FanRec r;
-    r.fo = fan_off[fe.u] + fe.i0;
+    r.fo = fan_off[fe.u] + fe.i0 + (int64_t)fe.j0 * u.rowlen;
     r.rp = u.rel + fe.i0;
-    r.rs = rowoff[u.s] + u.seg0;
+    r.rs = rowoff[u.s] + u.seg0 + fe.j0;
     r.rowlen = u.rowlen;
     r.ni = (int16_t)(fe.i1 - fe.i0);
-    r.seglen = (int16_t)u.seglen;
+    r.seglen = (int16_t)(fe.j1 - fe.j0);
     rec[k] = r;
   }
 }
@@ -2410,7 +2474,7 @@ cudaError_t launch_fanrec(const FanEnt* ent, int64_t n, const UTask* ut, const i
 
 cudaError_t launch_factor(bool fp32, const FactorArgs& a, int grid, size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<FactorArgs*>(&a)};
-  return cudaLaunchKernel(factor_fn(fp32, a.mma_mode, a.fan_ptr != nullptr, a.fuse_w > 0), dim3(grid), dim3(kFactorThreads), args,
+  return cudaLaunchKernel(factor_fn(fp32, a.mma_mode, a.gat != nullptr, a.fuse_w > 0), dim3(grid), dim3(kFactorThreads), args,
                           smem, st);
 }
 

@@ -60,34 +60,36 @@ struct Sim {
   double* panel(int s) { return pool.data() + P.valoff[s]; }
   int width(int s) const { return P.fcol[s + 1] - P.fcol[s]; }
 
-  // Fan-in mode: add the buffered updates into rows [r0, r1) of panel t, whose
-  // pieces start at piece pc0, in the lists' order.
-  void gather(int t, int pc0, int r0, int r1) {
+  // Fan-in mode: add the buffered updates of gather task G into columns
+  // [c0, c1) of rows [p0, p1) of panel t, in its list's order.
+  void gather(int t, const GatherTask& G, int p0, int p1) {
     const int ft = P.fcol[t], ldt = P.ld[t], rt = P.nrows[t];
     const int32_t* Rt = P.rows.data() + P.rowoff[t];
     double* T = panel(t);
-    for (int pc = pc0, p0 = r0; p0 < r1; ++pc, p0 += kFanPieceRows) {
-      const int p1 = std::min(r1, p0 + kFanPieceRows);
-      for (int64_t e = P.fan_ptr[pc]; e < P.fan_ptr[pc + 1]; ++e) {
-        const FanEnt& fe = P.fan_ent[e];
-        const UTask& u = P.ut[fe.u];
-        const int32_t* Rs = P.rows.data() + P.rowoff[u.s];
-        const double* F = fan.data() + P.fan_off[fe.u];
-        if (u.t != t || fe.i0 < 0 || fe.i0 >= fe.i1 || fe.i1 > u.rowlen) {
-          info = -1;  // inconsistent list
+    for (int64_t e = G.e0; e < G.e1; ++e) {
+      const FanEnt& fe = P.fan_ent[e];
+      const UTask& u = P.ut[fe.u];
+      const int32_t* Rs = P.rows.data() + P.rowoff[u.s];
+      const double* F = fan.data() + P.fan_off[fe.u];
+      if (u.t != t || fe.i0 < 0 || fe.i0 >= fe.i1 || fe.i1 > u.rowlen || fe.j0 < 0 || fe.j0 >= fe.j1 ||
+          fe.j1 > u.seglen) {
+        info = -1;  // inconsistent list
+        return;
+      }
+      for (int i = fe.i0; i < fe.i1; ++i) {
+        const int gi = Rs[u.row0 + i];
+        const int pos = (int)(std::lower_bound(Rt, Rt + rt, gi) - Rt);
+        if (pos < p0 || pos >= p1 || Rt[pos] != gi) {
+          info = -1;  // the row is not in this piece
           return;
         }
-        for (int i = fe.i0; i < fe.i1; ++i) {
-          const int gi = Rs[u.row0 + i];
-          const int pos = (int)(std::lower_bound(Rt, Rt + rt, gi) - Rt);
-          if (pos < p0 || pos >= p1 || Rt[pos] != gi) {
-            info = -1;  // the row is not in this piece
+        for (int j = fe.j0; j < fe.j1; ++j) {
+          const int gj = Rs[u.seg0 + j];
+          if (gj - ft < G.c0 || gj - ft >= G.c1) {
+            info = -1;  // the column is not in the task's window
             return;
           }
-          for (int j = 0; j < u.seglen; ++j) {
-            const int gj = Rs[u.seg0 + j];
-            if (gi >= gj) T[pos + (size_t)(gj - ft) * ldt] += F[i + (size_t)j * u.rowlen];
-          }
+          if (gi >= gj) T[pos + (size_t)(gj - ft) * ldt] += F[i + (size_t)j * u.rowlen];
         }
       }
     }
@@ -172,6 +174,12 @@ int spchol_plan_build(int64_t n, const int64_t* colptr, const int32_t* rowind, c
     return rc;
   }
   *out = p;
+  return 0;
+}
+
+int spchol_plan_split_gathers(spchol_plan_t p, int64_t max_values) {
+  if (!p) return -1;
+  split_gathers(p->plan, max_values >= 0 ? max_values : kGatherValues);
   return 0;
 }
 
@@ -321,7 +329,8 @@ int spchol_plan_simulate(spchol_plan_t p, const double* values, double* B, int64
     ++done;
     const bool skip = sim.info != 0;
     if (task >= gat0) {  // gather task (fan-in mode): one row piece of a panel
-      const int pc = P.gat_pc[task - gat0], o = P.pc_owner[pc];
+      const GatherTask& G = P.gat[task - gat0];
+      const int pc = G.pc, o = P.pc_owner[pc];
       const int t = o < ns ? o : P.trsm_sn[o - ns];
       const int w = sim.width(t);
       int p0, p1;
@@ -333,7 +342,7 @@ int spchol_plan_simulate(spchol_plan_t p, const double* values, double* B, int64
         p0 = r0 + (pc - P.fan_task[o]) * kFanPieceRows;
         p1 = std::min(std::min(P.nrows[t], r0 + tr), p0 + kFanPieceRows);
       }
-      if (!skip) sim.gather(t, pc, p0, p1);
+      if (!skip) sim.gather(t, G, p0, p1);
       if (o < ns) {
         if (--gd[t] < 0) return SPCHOL_EINTERNAL;
         if (gd[t] == 0) push(true, t);

@@ -75,14 +75,13 @@ struct FactorArgs {
   // panel-solve tiles + its predecessor)
   const int32_t* u_next;
   int32_t* u_dep;
-  // fan-in mode (null otherwise, see Plan::fan_ptr): the update tiles' private
+  // fan-in mode (null otherwise, see Plan::gat): the update tiles' private
   // buffers (panel type), each tile's offset in them, the first piece of each
   // diagonal / panel-solve task, the pieces' gather lists, and how many values
   // one gather batch stages in shared memory
   void* fan_buf;
   const int64_t* fan_off;
   const int32_t* fan_task;
-  const int64_t* fan_ptr;
   const FanRec* fan_rec;
   int32_t fan_cap;
   // its gather tasks (Plan::gat_first): ids gat0 + g (INT32_MAX: none), each
@@ -90,7 +89,7 @@ struct FactorArgs {
   // initial and live gather counts and the panel-solve tiles' live counters
   int32_t gat0;
   const int32_t* gat_first;
-  const int32_t* gat_pc;
+  const GatherTask* gat;
   const int32_t* pc_owner;
   const int32_t* gdiag0;
   int32_t* gdiag;

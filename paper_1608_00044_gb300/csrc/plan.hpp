@@ -111,10 +111,19 @@ constexpr int kWMaxWidth = 64;
 constexpr int kFanPieceRows = 32;
 
 // One entry of a fan-in gather list: rows [i0, i1) of update tile u fall in the
-// piece that owns the list.
+// piece that owns the list; its columns [j0, j1) are listed (all of the tile's,
+// or those in the window of a split gather).
 struct FanEnt {
   int32_t u;
-  int16_t i0, i1;
+  int16_t i0, i1, j0, j1;
+};
+
+// One gather task of the fan-in mode: list entries [e0, e1), which add into
+// columns [c0, c1) of piece pc.
+struct GatherTask {
+  int64_t e0, e1;
+  int32_t pc;
+  int16_t c0, c1;
 };
 
 struct Plan {
@@ -226,6 +235,7 @@ struct Plan {
   std::vector<int32_t> fan_task;  // ns + n_trsm
   std::vector<int64_t> fan_ptr;   // pieces + 1
   std::vector<FanEnt> fan_ent;
+  std::vector<int64_t> pc_values;  // pieces: the values their lists add
   // The solves of the fan-in mode: forward tile k stores its product (its
   // rows x nrhs, negated) at st_zf[k] * nrhs of one buffer and backward tile k
   // its product (its panel's width x nrhs) at st_zb[k] * nrhs of another,
@@ -238,12 +248,13 @@ struct Plan {
   // updates in one fixed order -- the order of the static chains.
   // Gather tasks (fan-in mode): one per row piece that receives updates, task
   // id ns + n_trsm + n_u + n_sub + g for g in [gat_first[t], gat_first[t + 1])
-  // of panel t, piece gat_pc[g], all made ready when the panel's last update
+  // of panel t, piece gat[g].pc, all made ready when the panel's last update
   // tile lands.  pc_owner[piece]: the task whose rows it holds (t: the
   // diagonal task, ns + k: panel-solve tile k).  The diagonal task waits for
   // its gathers (gdiag0[t] of them; none: it is ready with the updates), each
   // panel-solve tile for the diagonal task and its own gathers (tdep0[k]).
-  std::vector<int32_t> gat_first, gat_pc, pc_owner, gdiag0, tdep0;
+  std::vector<int32_t> gat_first, pc_owner, gdiag0, tdep0;
+  std::vector<GatherTask> gat;
   int32_t n_gat = 0;
   std::vector<int64_t> st_zf, st_zb;  // n_st + 1
   // the forward gather's record of each rt_tile entry: the tile's buffer (in
@@ -277,6 +288,18 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
 // that stay within max_steps; the panels above those become tasks of their
 // own.  Not after the warp-level launches have been laid out (Plan::wsub).
 void split_subtrees(Plan& plan, int64_t max_steps);
+
+// Split the gather tasks that add more than max_values values (fan-in mode)
+// into column windows of a multiple of 8 columns, each with a list of its own
+// (appended to fan_ent): gathers of one piece add into disjoint columns, so
+// every entry still receives its updates in the piece's list order.  A gather
+// adds its tiles one after another, and near the root -- 300 tiles and 100,000
+// values a piece, one panel after another, the chip idle -- those were most of
+// the critical path (300 us each).  Factorization of a 27^3 Laplacian: no
+// split 11.8 ms, at 16384 values 8.6, 8192 8.0, 4096 7.8, 2048 7.8 (and more
+// list entries the finer: 0.50, 0.61, 0.71, 0.84 and 1.02 million, which the analysis makes).
+constexpr int64_t kGatherValues = 8192;
+void split_gathers(Plan& plan, int64_t max_values);
 
 // The GPU launch's max_steps: a CTA's average share of all steps (kPlanCtas)
 // over kSubtreeShare.  A subtree task runs its steps one after

@@ -560,7 +560,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
         const int32_t pc = piece_of(U.t, p, end);
         const int32_t i1 =
             end >= rt ? U.rowlen : (int32_t)(std::lower_bound(Rs + i, Rs + U.rowlen, Rt[end]) - Rs);
-        items.push_back(Item{pc, FanEnt{u, (int16_t)i, (int16_t)i1}});
+        items.push_back(Item{pc, FanEnt{u, (int16_t)i, (int16_t)i1, 0, (int16_t)U.seglen}});
         i = i1;
       }
     }
@@ -568,9 +568,15 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     P.fan_ptr.assign((size_t)npc + 1, 0);
     for (const Item& it : items) P.fan_ptr[it.pc + 1]++;
     for (int32_t k = 0; k < npc; ++k) P.fan_ptr[k + 1] += P.fan_ptr[k];
+    P.fan_ent.reserve(2 * items.size());  // split_gathers appends
     P.fan_ent.resize(items.size());
+    std::vector<int64_t> values(npc, 0);
     std::vector<int64_t> fill(P.fan_ptr.begin(), P.fan_ptr.end() - 1);
-    for (const Item& it : items) P.fan_ent[fill[it.pc]++] = it.e;
+    for (const Item& it : items) {
+      P.fan_ent[fill[it.pc]++] = it.e;
+      values[it.pc] += (int64_t)(it.e.i1 - it.e.i0) * (it.e.j1 - it.e.j0);
+    }
+    P.pc_values.swap(values);
   }
 
   // ---- subtree tasks ------------------------------------------------------------
@@ -638,7 +644,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     }
   // ---- gather tasks of the fan-in mode (see Plan::gat_first) ---------------------
   P.gat_first.clear();
-  P.gat_pc.clear();
+  P.gat.clear();
   P.pc_owner.clear();
   P.gdiag0.clear();
   P.tdep0.clear();
@@ -660,11 +666,11 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     P.tdep0.assign(P.n_trsm, 1);
     for (int32_t s = 0; s < ns; ++s) {
       // a panel's pieces are numbered consecutively, from its diagonal block's
-      P.gat_first[s] = (int32_t)P.gat_pc.size();
+      P.gat_first[s] = (int32_t)P.gat.size();
       const int32_t pc_end = s + 1 < ns ? P.fan_task[s + 1] : npc;
       for (int32_t pc = P.fan_task[s]; pc < pc_end; ++pc)
         if (P.fan_ptr[pc + 1] > P.fan_ptr[pc]) {
-          P.gat_pc.push_back(pc);
+          P.gat.push_back(GatherTask{P.fan_ptr[pc], P.fan_ptr[pc + 1], pc, 0, (int16_t)(P.fcol[s + 1] - P.fcol[s])});
           const int32_t o = P.pc_owner[pc];
           if (o < ns)
             P.gdiag0[s]++;
@@ -672,8 +678,8 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
             P.tdep0[o - ns]++;
         }
     }
-    P.gat_first[ns] = (int32_t)P.gat_pc.size();
-    P.n_gat = (int32_t)P.gat_pc.size();
+    P.gat_first[ns] = (int32_t)P.gat.size();
+    P.n_gat = (int32_t)P.gat.size();
     P.n_task_ids += P.n_gat;
     P.n_factor_tasks += P.n_gat;
     P.n_hi_tasks += P.n_gat;
@@ -861,6 +867,67 @@ void split_subtrees(Plan& P, int64_t max_steps) {
   P.sub_hi.swap(hi);
   P.in_sub.swap(in);
   P.wsub.clear();  // the warp-level launches take the tasks as they were
+}
+
+void split_gathers(Plan& P, int64_t max_values) {
+  if (P.n_gat == 0) return;
+  struct Left {  // a tile's columns that no window has had yet
+    const int32_t* cols;
+    int32_t next;
+    int16_t j;
+  };
+  std::vector<Left> left;
+  std::vector<GatherTask> gat;
+  gat.reserve(2 * P.gat.size());
+  for (int32_t s = 0; s < P.ns; ++s) {
+    const int32_t g0 = P.gat_first[s], g1 = P.gat_first[s + 1], f = P.fcol[s], w = P.fcol[s + 1] - f;
+    P.gat_first[s] = (int32_t)gat.size();
+    for (int32_t g = g0; g < g1; ++g) {
+      const GatherTask G = P.gat[g];
+      const int64_t parts = std::min<int64_t>((P.pc_values[G.pc] + max_values - 1) / std::max<int64_t>(max_values, 1), (w + 7) / 8);
+      if (parts <= 1 || G.c0 != 0 || G.c1 != w) {
+        gat.push_back(G);
+        continue;
+      }
+      const int32_t wide = (int32_t)(((w + parts - 1) / parts + 7) / 8 * 8), o = P.pc_owner[G.pc];
+      left.clear();
+      for (int64_t e = G.e0; e < G.e1; ++e) {
+        const UTask& u = P.ut[P.fan_ent[e].u];
+        const int32_t* cols = P.rows.data() + P.rowoff[u.s] + u.seg0;  // ascending
+        left.push_back(Left{cols, cols[0], 0});
+      }
+      int32_t n = 0;
+      for (int32_t c0 = 0; c0 < w; c0 += wide) {
+        const int32_t c1 = std::min(w, c0 + wide);
+        const int64_t e0 = (int64_t)P.fan_ent.size();
+        for (int64_t e = G.e0; e < G.e1; ++e) {
+          FanEnt fe = P.fan_ent[e];
+          Left& l = left[e - G.e0];  // the tile's columns from here on lie at c0 or beyond
+          const int32_t end = f + c1;
+          if (l.next >= end) continue;
+          fe.j0 = l.j;
+          int16_t j = l.j + 1;
+          while (j < fe.j1 && l.cols[j] < end) ++j;
+          l.j = j;
+          l.next = j < fe.j1 ? l.cols[j] : INT32_MAX;
+          fe.j1 = j;
+          P.fan_ent.push_back(fe);
+        }
+        const int64_t e1 = (int64_t)P.fan_ent.size();
+        if (e0 == e1) continue;  // no tile has a column there
+        gat.push_back(GatherTask{e0, e1, G.pc, (int16_t)c0, (int16_t)c1});
+        ++n;
+      }
+      (o < P.ns ? P.gdiag0[o] : P.tdep0[o - P.ns]) += n - 1;
+    }
+  }
+  P.gat_first[P.ns] = (int32_t)gat.size();
+  const int32_t more = (int32_t)gat.size() - P.n_gat;
+  P.n_gat += more;
+  P.n_task_ids += more;
+  P.n_factor_tasks += more;
+  P.n_hi_tasks += more;
+  P.gat.swap(gat);
 }
 
 }  // namespace spchol

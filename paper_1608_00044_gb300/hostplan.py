@@ -18,6 +18,7 @@ HOST_LIB_PATH = os.path.join(_HERE, "libspchol_host.so")
 _vp = ctypes.c_void_p
 SIGNATURES = [
     ("spchol_plan_build", ctypes.c_int, [ctypes.c_int64, _vp, _vp, _vp, ctypes.POINTER(Options), ctypes.POINTER(_vp)]),
+    ("spchol_plan_split_gathers", ctypes.c_int, [_vp, ctypes.c_int64]),
     ("spchol_plan_split_subtrees", ctypes.c_int, [_vp, ctypes.c_int64]),
     ("spchol_plan_len", ctypes.c_int64, [_vp, ctypes.c_int]),
     ("spchol_plan_get", ctypes.c_int, [_vp, ctypes.c_int, _vp]),
@@ -77,6 +78,12 @@ class HostPlan:
     def split_subtrees(self, max_steps: int = -1) -> None:
         """Cut the subtree tasks as the GPU library's analyze does (max_steps < 0: at its own limit)."""
         rc = load().spchol_plan_split_subtrees(self._h, int(max_steps))
+        if rc != 0:
+            raise ValueError(rc)
+
+    def split_gathers(self, max_values: int = -1) -> None:
+        """Split the fan-in gathers as the GPU library's analyze does (max_values < 0: at its own limit)."""
+        rc = load().spchol_plan_split_gathers(self._h, int(max_values))
         if rc != 0:
             raise ValueError(rc)
 

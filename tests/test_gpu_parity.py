@@ -958,3 +958,29 @@ def test_diagonal_tasks_that_solve_their_rows(name, W, precision, deterministic)
     spchol.destroy(h)
     assert d <= (1e-11 if precision == "FP64" else 1e-5) * lmax, (d, lmax)
     assert oracle.berr(A, X, b) <= (BERR_FP64 if precision == "FP64" else 1e-12)
+
+
+@pytest.mark.parametrize("precision", [spchol.FP64, spchol.FP32])
+@pytest.mark.parametrize("name,W", [("lap3d_20", 64), ("lap3d_20", 128), ("diff3d_9", 8), ("lap2d_64", 9)])
+def test_split_fanin_gathers_are_bitwise_the_static_order(name, W, precision):
+    """Gathers split into column windows, the threads' own entries (up to 8
+    columns) and the wider pieces: bit for bit the static chains' factor, seen
+    through the FP64 solution (FP32: through the refined one, whose every
+    iterate the factor decides)."""
+    from paper_1608_00044_gb300 import hostplan as hp
+
+    A, perm, b = gridgen.workload(name)
+    P = hp.HostPlan(A.n, A.colptr, A.rowind, perm, max_width=W, deterministic=2)
+    before = P.scalars()["factor_tasks"]
+    P.split_gathers()
+    if name.startswith("lap3d"):
+        assert P.scalars()["factor_tasks"] > before
+    P.close()
+    B = gridgen.rhs_uniform(A.n, 2, seed=4)
+    X = []
+    for det in (1, 2):
+        rc, Xd, st, h = gpu_factor_solve(A, perm, B, deterministic=det, max_width=W, precision=precision)
+        assert rc == 0
+        spchol.destroy(h)
+        X.append(Xd)
+    np.testing.assert_array_equal(X[0], X[1])

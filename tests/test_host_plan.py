@@ -484,3 +484,29 @@ def test_split_subtrees_are_maximal_and_run_the_protocol(name, W, max_steps):
     # the order of the sums alone differs: at most a few hundred roundings of the largest entry
     assert np.abs(pool - pool0).max() <= 1e-13 * np.abs(pool0).max()
     assert oracle.berr(A, X, b) <= 1e-14
+
+
+@pytest.mark.parametrize("name,W,max_values", [("lap3d_12", 64, 1), ("lap3d_12", 64, 300), ("diff3d_9", 16, 64),
+                                               ("lap2d_24", 128, 40), ("lap3d_20", 64, -1)])
+def test_split_gathers_keep_the_order_of_every_entry(name, W, max_values):
+    """Fan-in gathers split at max_values values: the lists of the pieces
+    unchanged, the tasks counted again -- and the simulator, which rejects a
+    column outside its task's window, runs the split plan to the unsplit plan's
+    factor and solution bit for bit."""
+    A, perm, b = gridgen.workload(name)
+    P, Q = _plan(A, perm, deterministic=2, max_width=W), _plan(A, perm, deterministic=2, max_width=W)
+    Q.split_gathers(max_values)
+    ptr = P.get(hp.FANPTR)
+    assert np.array_equal(ptr, Q.get(hp.FANPTR))
+    assert np.array_equal(P.get(hp.FANENT), Q.get(hp.FANENT)[:3 * ptr[-1]])
+    more = Q.scalars()["factor_tasks"] - P.scalars()["factor_tasks"]
+    assert more >= 0 and more == Q.scalars()["n_hi_tasks"] - P.scalars()["n_hi_tasks"]
+    if max_values > 0:
+        assert more > 0
+    B = b[:, None]
+    want = P.simulate(A.values, B, seed=0, want_pool=True)
+    for seed in (1, 2):
+        got = Q.simulate(A.values, B, seed=seed, want_pool=True)
+        assert got[0] == 0
+        np.testing.assert_array_equal(got[1], want[1])
+        np.testing.assert_array_equal(got[2], want[2])
