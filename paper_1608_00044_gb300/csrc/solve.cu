@@ -399,9 +399,14 @@ __device__ __forceinline__ void oz_stage_ys(const SolveArgs& a, const OzBuf& b, 
 // kSolveFanBatch list entries at a time: warp 0 cuts the batch where its
 // values would overflow the staging area (the entries' records were fetched
 // during the previous batch); all threads load the batch's values (eight
-// loads in flight each) and map each entry's rows to the panel's columns;
-// then each thread adds, for the (column, right-hand side) entries it owns,
-// the batch's values in order from shared memory.  Backward: the panel's own
+// loads in flight each), and a warp per entry maps its rows to the panel's
+// columns; then each thread adds, for the (column, right-hand side) entries it
+// owns, the batch's values in order from shared memory, four entries' read
+// ahead.  What bounds it is latency, one panel of the top separators after
+// another: their tasks take 90 us on a 27^3 Laplacian with 2 right-hand sides
+// (110 with the map made one (entry, column) pair a thread, and the values read
+// one at a time), the whole solve 3.65 ms (3.79).  The next batch's rows and
+// values in registers while one is added spilled: 5.2 ms.  Backward: the panel's own
 // tiles, each thread summing its entries' values over the tiles in order.
 using SolveFanRec = Plan::SolveFanRec;
 constexpr int kSolveFanBatch = 32;
@@ -417,7 +422,8 @@ constexpr size_t solve_fan_smem_bytes(int max_w) {
 }
 
 __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, int r0, int nrc, unsigned char* ex) {
-  const int tid = threadIdx.x, nt = blockDim.x;
+  constexpr int kWarps = kSolveThreads / 32, kEnt = kSolveFanBatch / kWarps, kAhead = 4;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   SolveFanMeta* meta = reinterpret_cast<SolveFanMeta*>(ex);
   int* scal = reinterpret_cast<int*>(meta + kSolveFanBatch);  // entries and values of the batch
   int16_t* inv = reinterpret_cast<int16_t*>(scal + 4);        // [batch entry][column]: its row, or -1
@@ -429,7 +435,6 @@ __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, 
   if (tid < 32 && e1 - 1 - tid >= e0) rec = a.rt_rec[e1 - 1 - tid];
   for (int eb = e1; eb > e0;) {
     __syncthreads();  // the right-hand sides are staged, or the previous batch is added
-    for (int idx = tid; idx < kSolveFanBatch * w; idx += nt) inv[idx] = -1;
     if (tid < 32) {
       const bool have = eb - 1 - tid >= e0;
       const int n = have ? rec.ni * nrc : 0;
@@ -464,18 +469,15 @@ __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, 
       if (tid == 0) atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);
       total = 0;
     }
-    // the entries' rows mapped to the panel's columns ...
-    for (int idx = tid; idx < nb * w; idx += nt) {
-      const int b = idx / w, i = idx - b * w;
-      if (i < meta[b].ni) {
-        const int c = __ldg(a.pv.rows + meta[b].ro + i) - f;
-        if (c >= 0 && c < w)
-          inv[b * w + c] = (int16_t)i;
-        else
-          atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);
-      }
+    // the entries' rows, a warp per entry (the first 32 of each on their way
+    // while the values are loaded) ...
+    int row[kEnt];
+#pragma unroll
+    for (int q = 0; q < kEnt; ++q) {
+      const int b = warp + q * kWarps;
+      row[q] = b < nb && lane < meta[b].ni ? __ldg(a.pv.rows + meta[b].ro + lane) : 0;
     }
-    // ... and their values, eight loads in flight per thread
+    // ... their values, eight loads in flight per thread ...
     for (int v0 = 0; v0 < total; v0 += 8 * nt) {
       double v[8];
 #pragma unroll
@@ -499,13 +501,37 @@ __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, 
         if (idx < total) Bv[idx] = v[u];
       }
     }
+    // ... and the map from the panel's columns to them
+#pragma unroll
+    for (int q = 0; q < kEnt; ++q) {
+      const int b = warp + q * kWarps;
+      if (b >= nb) break;  // the same in every lane
+      const int ni = meta[b].ni;
+      for (int c = lane; c < w; c += 32) inv[b * w + c] = -1;
+      __syncwarp();
+      for (int i = lane; i < ni; i += 32) {
+        const int c = (i == lane ? row[q] : __ldg(a.pv.rows + meta[b].ro + i)) - f;
+        if (c >= 0 && c < w)
+          inv[b * w + c] = (int16_t)i;
+        else
+          atomicCAS(&a.ctrl[kErr], 0, SPCHOL_DEV_EINTERNAL);
+      }
+    }
     __syncthreads();
     for (int p = tid; p < w * nrc; p += nt) {
       const int c = p % w, r = p / w;
       double y = Ys[p];
-      for (int b = 0; b < nb; ++b) {
-        const int i = inv[b * w + c];
-        if (i >= 0) y += Bv[meta[b].pre + r * meta[b].ni + i];
+      for (int b0 = 0; b0 < nb; b0 += kAhead) {
+        int i[kAhead];
+        double x[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) i[u] = b0 + u < nb ? inv[(b0 + u) * w + c] : -1;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          x[u] = i[u] >= 0 ? Bv[meta[b0 + u].pre + r * meta[b0 + u].ni + i[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (i[u] >= 0) y += x[u];
       }
       Ys[p] = y;
     }
