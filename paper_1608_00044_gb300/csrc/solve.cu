@@ -401,13 +401,15 @@ __device__ __forceinline__ void oz_stage_ys(const SolveArgs& a, const OzBuf& b, 
 // during the previous batch); all threads load the batch's values (eight
 // loads in flight each), and a warp per entry maps its rows to the panel's
 // columns; then each thread adds, for the (column, right-hand side) entries it
-// owns, the batch's values in order from shared memory, four entries' read
-// ahead.  What bounds it is latency, one panel of the top separators after
-// another: their tasks take 90 us on a 27^3 Laplacian with 2 right-hand sides
-// (110 with the map made one (entry, column) pair a thread, and the values read
-// one at a time), the whole solve 3.65 ms (3.79).  The next batch's rows and
-// values in registers while one is added spilled: 5.2 ms.  Backward: the panel's own
-// tiles, each thread summing its entries' values over the tiles in order.
+// owns, the batch's values in order from shared memory.  What bounds it is
+// latency with few right-hand sides, one panel of the top separators after
+// another, and the FP64 pipe with many.  Solve of a 27^3 Laplacian with 1 / 4 /
+// 16 right-hand sides: 3.15 / 3.92 / 10.4 ms (3.28 / 3.99 / 10.6 with the map
+// made one (entry, column) pair a thread).  Four entries' values read ahead
+// were slower (3.33 / 4.05, and 10.8 where the adds were predicated), and so
+// was the next batch in registers, which spilled (5.2 ms with 2).
+// Backward: the panel's own tiles, each thread summing its entries' values over
+// the tiles in order.
 using SolveFanRec = Plan::SolveFanRec;
 constexpr int kSolveFanBatch = 32;
 constexpr int kSolveFanVals = 2048;  // staged values per batch (an entry has at most 64 x 8)
@@ -422,7 +424,7 @@ constexpr size_t solve_fan_smem_bytes(int max_w) {
 }
 
 __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, int r0, int nrc, unsigned char* ex) {
-  constexpr int kWarps = kSolveThreads / 32, kEnt = kSolveFanBatch / kWarps, kAhead = 4;
+  constexpr int kWarps = kSolveThreads / 32, kEnt = kSolveFanBatch / kWarps;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   SolveFanMeta* meta = reinterpret_cast<SolveFanMeta*>(ex);
   int* scal = reinterpret_cast<int*>(meta + kSolveFanBatch);  // entries and values of the batch
@@ -521,17 +523,11 @@ __device__ void fwd_gather(const SolveArgs& a, int s, int f, int w, double* Ys, 
     for (int p = tid; p < w * nrc; p += nt) {
       const int c = p % w, r = p / w;
       double y = Ys[p];
-      for (int b0 = 0; b0 < nb; b0 += kAhead) {
-        int i[kAhead];
-        double x[kAhead];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) i[u] = b0 + u < nb ? inv[(b0 + u) * w + c] : -1;
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u)
-          x[u] = i[u] >= 0 ? Bv[meta[b0 + u].pre + r * meta[b0 + u].ni + i[u]] : 0.0;
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u)
-          if (i[u] >= 0) y += x[u];
+      // (a branch per entry: an add with every lane predicated off would hold
+      // the FP64 pipe as long as any)
+      for (int b = 0; b < nb; ++b) {
+        const int i = inv[b * w + c];
+        if (i >= 0) y += Bv[meta[b].pre + r * meta[b].ni + i];
       }
       Ys[p] = y;
     }
