@@ -50,7 +50,12 @@ enum {
   SPCHOL_PLAN_FANOFF = 18,   /* n_u+1: offset of each update tile's private buffer (values) */
   SPCHOL_PLAN_FANTASK = 19,  /* ns+n_trsm: first row piece of each diagonal task, then of each panel-solve tile */
   SPCHOL_PLAN_FANPTR = 20,   /* pieces+1: offsets into FANENT */
-  SPCHOL_PLAN_FANENT = 21    /* 3 * entries: (update tile, first row, end row) per gather-list entry */
+  SPCHOL_PLAN_FANENT = 21,   /* 3 * entries: (update tile, first row, end row) per entry of the pieces' lists */
+  SPCHOL_PLAN_GATHERS = 22,  /* 5 * gather tasks: (first entry, end entry, piece, first column, end column):
+                                entries of GATENT, columns of the panel */
+  SPCHOL_PLAN_GATENT = 23    /* 5 * entries: (update tile, first row, end row, first column, end column of the
+                                tile) per entry of the gather tasks' lists: the pieces' lists, cut into
+                                column windows once the gathers are split */
 };
 
 /* Host-only analysis; same arguments and return codes as spchol_analyze. */

@@ -383,7 +383,11 @@ int setup_device(spchol_handle_t h) {
   // the others run on CTAs, none longer than a fair share of the launch (the
   // fault injection withholds the flop budget's task of the root)
   if (!warp_sub && h->opt.fault_inject == 0) split_subtrees(P, subtree_step_budget(P));
-  if (P.params.fanin && h->opt.fault_inject == 0) split_gathers(P, kGatherValues);
+  if (P.params.fanin && h->opt.fault_inject == 0) {
+    split_gathers(P, kGatherValues);
+    if (!P.gat_ent.empty()) std::vector<FanEnt>().swap(P.fan_ent);  // the cut lists take its place
+  }
+  const std::vector<FanEnt>& fan_ent = gather_entries(P);
   Arena& A = h->arena;
   auto r32 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int32_t)); };
   auto r64 = [&](size_t n) { return A.reserve(std::max<size_t>(n, 1) * sizeof(int64_t)); };
@@ -463,7 +467,7 @@ int setup_device(spchol_handle_t h) {
          o_fdd = det ? r32(P.ft_dep0.size()) : 0;
   const bool fan = P.params.fanin;
   size_t o_fano = fan ? r64(P.fan_off.size()) : 0, o_fant = fan ? r32(P.fan_task.size()) : 0,
-         o_fane = fan ? A.reserve(std::max<size_t>(P.fan_ent.size(), 1) * sizeof(FanEnt)) : 0,
+         o_fane = fan ? A.reserve(std::max<size_t>(fan_ent.size(), 1) * sizeof(FanEnt)) : 0,
          o_stzf = fan ? r64(P.st_zf.size()) : 0, o_stzb = fan ? r64(P.st_zb.size()) : 0,
          o_rtrec = fan ? A.reserve(std::max<size_t>(P.rt_rec.size(), 1) * sizeof(Plan::SolveFanRec)) : 0,
          o_gatf = fan ? r32(P.gat_first.size()) : 0, o_gatp = fan ? A.reserve(std::max<size_t>(P.gat.size(), 1) * sizeof(GatherTask)) : 0,
@@ -633,7 +637,7 @@ int setup_device(spchol_handle_t h) {
               (rc = upload(h, h->d_ft_dep0, P.ft_dep0))))
     return rc;
   if (fan && ((rc = upload(h, h->d_fan_off, P.fan_off)) || (rc = upload(h, h->d_fan_task, P.fan_task)) ||
-              (rc = upload(h, h->d_fan_ent, P.fan_ent)) ||
+              (rc = upload(h, h->d_fan_ent, fan_ent)) ||
               (rc = upload(h, h->d_st_zf, P.st_zf)) || (rc = upload(h, h->d_st_zb, P.st_zb)) ||
               (rc = upload(h, h->d_gat_first, P.gat_first)) || (rc = upload(h, h->d_gat, P.gat)) ||
               (rc = upload(h, h->d_pc_owner, P.pc_owner)) || (rc = upload(h, h->d_gdiag0, P.gdiag0)) ||
@@ -644,8 +648,8 @@ int setup_device(spchol_handle_t h) {
     // + 16 bytes: the gather copies whole 16-byte pieces, up to one past the last value
     h->fan_buf_bytes = std::max<size_t>((((size_t)P.fan_off.back() * esz + 15) & ~size_t(15)) + 16, 256);
     DALLOC(h->d_fan_buf, h->fan_buf_bytes, nullptr);
-    DALLOC(h->d_fan_rec, std::max<size_t>(P.fan_ent.size(), 1) * sizeof(FanRec), nullptr);
-    CU(launch_fanrec(h->d_fan_ent, (int64_t)P.fan_ent.size(), h->d_ut, h->d_fan_off, h->d_rowoff, h->d_fan_rec,
+    DALLOC(h->d_fan_rec, std::max<size_t>(fan_ent.size(), 1) * sizeof(FanRec), nullptr);
+    CU(launch_fanrec(h->d_fan_ent, (int64_t)fan_ent.size(), h->d_ut, h->d_fan_off, h->d_rowoff, h->d_fan_rec,
                      g_upload_stream));
   }
   h->pool_bytes = std::max<size_t>((size_t)P.valoff[ns] * esz, 256);
@@ -712,7 +716,7 @@ int setup_device(spchol_handle_t h) {
                                        (size_t)P.n_w * (h->fp32 ? sizeof(float) : sizeof(double)) +
                                        (size_t)P.n_rel * sizeof(int32_t) + (size_t)P.ns * (h->d_tmaps ? 128 : 0) +
                                        (oz ? (size_t)P.sliceoff[ns] * sizeof(uint16_t) : 0) + h->fan_buf_bytes +
-                                       (h->d_fan_rec ? P.fan_ent.size() * sizeof(FanRec) : 0));
+                                       (h->d_fan_rec ? fan_ent.size() * sizeof(FanRec) : 0));
   h->stats.grid_factor = h->grid_factor;
   h->stats.grid_solve = h->grid_solve;
   h->stats.tma_staging = h->d_tmaps != nullptr ? 1 : 0;

@@ -67,7 +67,7 @@ struct Sim {
     const int32_t* Rt = P.rows.data() + P.rowoff[t];
     double* T = panel(t);
     for (int64_t e = G.e0; e < G.e1; ++e) {
-      const FanEnt& fe = P.fan_ent[e];
+      const FanEnt& fe = gather_entries(P)[e];
       const UTask& u = P.ut[fe.u];
       const int32_t* Rs = P.rows.data() + P.rowoff[u.s];
       const double* F = fan.data() + P.fan_off[fe.u];
@@ -206,6 +206,8 @@ int64_t spchol_plan_len(spchol_plan_t p, int what) {
     case SPCHOL_PLAN_FANTASK: return (int64_t)P.fan_task.size();
     case SPCHOL_PLAN_FANPTR: return (int64_t)P.fan_ptr.size();
     case SPCHOL_PLAN_FANENT: return 3 * (int64_t)P.fan_ent.size();
+    case SPCHOL_PLAN_GATHERS: return 5 * (int64_t)P.gat.size();
+    case SPCHOL_PLAN_GATENT: return 5 * (int64_t)gather_entries(P).size();
     default: return -1;
   }
 }
@@ -244,6 +246,21 @@ int spchol_plan_get(spchol_plan_t p, int what, int64_t* dst) {
         dst[3 * i + 2] = P.fan_ent[i].i1;
       }
       break;
+    case SPCHOL_PLAN_GATHERS:
+      for (size_t i = 0; i < P.gat.size(); ++i) {
+        const GatherTask& G = P.gat[i];
+        int64_t* d = dst + 5 * i;
+        d[0] = G.e0; d[1] = G.e1; d[2] = G.pc; d[3] = G.c0; d[4] = G.c1;
+      }
+      break;
+    case SPCHOL_PLAN_GATENT: {
+      const std::vector<FanEnt>& ent = gather_entries(P);
+      for (size_t i = 0; i < ent.size(); ++i) {
+        int64_t* d = dst + 5 * i;
+        d[0] = ent[i].u; d[1] = ent[i].i0; d[2] = ent[i].i1; d[3] = ent[i].j0; d[4] = ent[i].j1;
+      }
+      break;
+    }
     case SPCHOL_PLAN_UTASKS:
       for (size_t i = 0; i < P.ut.size(); ++i) {
         const UTask& u = P.ut[i];

@@ -118,8 +118,8 @@ struct FanEnt {
   int16_t i0, i1, j0, j1;
 };
 
-// One gather task of the fan-in mode: list entries [e0, e1), which add into
-// columns [c0, c1) of piece pc.
+// One gather task of the fan-in mode: list entries [e0, e1) (gather_entries),
+// which add into columns [c0, c1) of piece pc.
 struct GatherTask {
   int64_t e0, e1;
   int32_t pc;
@@ -255,6 +255,7 @@ struct Plan {
   // panel-solve tile for the diagonal task and its own gathers (tdep0[k]).
   std::vector<int32_t> gat_first, pc_owner, gdiag0, tdep0;
   std::vector<GatherTask> gat;
+  std::vector<FanEnt> gat_ent;  // the tasks' lists once split_gathers has cut them; before, they are the pieces' own (fan_ent)
   int32_t n_gat = 0;
   std::vector<int64_t> st_zf, st_zb;  // n_st + 1
   // the forward gather's record of each rt_tile entry: the tile's buffer (in
@@ -289,15 +290,19 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
 // own.  Not after the warp-level launches have been laid out (Plan::wsub).
 void split_subtrees(Plan& plan, int64_t max_steps);
 
+// The lists that Plan::gat's tasks index.
+inline const std::vector<FanEnt>& gather_entries(const Plan& P) { return P.gat_ent.empty() ? P.fan_ent : P.gat_ent; }
+
 // Split the gather tasks that add more than max_values values (fan-in mode)
-// into column windows of a multiple of 8 columns, each with a list of its own
-// (appended to fan_ent): gathers of one piece add into disjoint columns, so
-// every entry still receives its updates in the piece's list order.  A gather
-// adds its tiles one after another, and near the root -- 300 tiles and 100,000
-// values a piece, one panel after another, the chip idle -- those were most of
-// the critical path (300 us each).  Factorization of a 27^3 Laplacian: no
-// split 11.8 ms, at 16384 values 8.6, 8192 8.0, 4096 7.8, 2048 7.8 (and more
-// list entries the finer: 0.50, 0.61, 0.71, 0.84 and 1.02 million, which the analysis makes).
+// into column windows of a multiple of 8 columns, each with a list of its own:
+// gathers of one piece add into disjoint columns, so every entry still receives
+// its updates in the piece's list order.  Every task's list is written to
+// Plan::gat_ent, one after another.  A gather adds its tiles one after another,
+// and near the root -- 300 tiles and 100,000 values a piece, one panel after
+// another, the chip idle -- those were most of the critical path (300 us each).
+// Factorization of a 27^3 Laplacian: no split 11.8 ms, at 16384 values 8.6, 8192
+// 8.0, 4096 7.8, 2048 7.8 (and more list entries the finer: 0.50, 0.61, 0.71,
+// 0.84 and 1.02 million, which the analysis makes).
 constexpr int64_t kGatherValues = 8192;
 void split_gathers(Plan& plan, int64_t max_values);
 

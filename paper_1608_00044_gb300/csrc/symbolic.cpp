@@ -498,6 +498,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
   P.fan_task.clear();
   P.fan_ptr.clear();
   P.fan_ent.clear();
+  P.gat_ent.clear();
   if (prm.fanin) {
     P.fan_off.assign((size_t)P.n_u + 1, 0);
     for (int32_t u = 0; u < P.n_u; ++u)
@@ -568,7 +569,6 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     P.fan_ptr.assign((size_t)npc + 1, 0);
     for (const Item& it : items) P.fan_ptr[it.pc + 1]++;
     for (int32_t k = 0; k < npc; ++k) P.fan_ptr[k + 1] += P.fan_ptr[k];
-    P.fan_ent.reserve(2 * items.size());  // split_gathers appends
     P.fan_ent.resize(items.size());
     std::vector<int64_t> values(npc, 0);
     std::vector<int64_t> fill(P.fan_ptr.begin(), P.fan_ptr.end() - 1);
@@ -871,14 +871,18 @@ void split_subtrees(Plan& P, int64_t max_steps) {
 
 void split_gathers(Plan& P, int64_t max_values) {
   if (P.n_gat == 0) return;
-  struct Left {  // a tile's columns that no window has had yet
-    const int32_t* cols;
-    int32_t next;
-    int16_t j;
-  };
-  std::vector<Left> left;
+  constexpr int64_t kAhead = 16;  // entries whose tile and columns are on their way
+  const std::vector<FanEnt>& all = gather_entries(P);
+  std::vector<std::vector<FanEnt>> win((P.max_w + 7) / 8);  // the lists of one gather's windows
+  std::vector<FanEnt> ent;
+  ent.reserve(2 * all.size() + all.size() / 2);
   std::vector<GatherTask> gat;
   gat.reserve(2 * P.gat.size());
+  auto put = [&](const GatherTask& G, const FanEnt* first, const FanEnt* last, int32_t c0, int32_t c1) {
+    const int64_t e0 = (int64_t)ent.size();
+    ent.insert(ent.end(), first, last);
+    gat.push_back(GatherTask{e0, (int64_t)ent.size(), G.pc, (int16_t)c0, (int16_t)c1});
+  };
   for (int32_t s = 0; s < P.ns; ++s) {
     const int32_t g0 = P.gat_first[s], g1 = P.gat_first[s + 1], f = P.fcol[s], w = P.fcol[s + 1] - f;
     P.gat_first[s] = (int32_t)gat.size();
@@ -886,36 +890,43 @@ void split_gathers(Plan& P, int64_t max_values) {
       const GatherTask G = P.gat[g];
       const int64_t parts = std::min<int64_t>((P.pc_values[G.pc] + max_values - 1) / std::max<int64_t>(max_values, 1), (w + 7) / 8);
       if (parts <= 1 || G.c0 != 0 || G.c1 != w) {
-        gat.push_back(G);
+        put(G, all.data() + G.e0, all.data() + G.e1, G.c0, G.c1);
         continue;
       }
       const int32_t wide = (int32_t)(((w + parts - 1) / parts + 7) / 8 * 8), o = P.pc_owner[G.pc];
-      left.clear();
+      // each entry once, cut at the windows' edges: a window's list keeps the
+      // piece's order
       for (int64_t e = G.e0; e < G.e1; ++e) {
-        const UTask& u = P.ut[P.fan_ent[e].u];
+        if (e + 2 * kAhead < G.e1) __builtin_prefetch(&P.ut[all[e + 2 * kAhead].u]);
+        if (e + kAhead < G.e1) {
+          const UTask& u = P.ut[all[e + kAhead].u];
+          __builtin_prefetch(P.rows.data() + P.rowoff[u.s] + u.seg0);
+        }
+        FanEnt fe = all[e];
+        const UTask& u = P.ut[fe.u];
         const int32_t* cols = P.rows.data() + P.rowoff[u.s] + u.seg0;  // ascending
-        left.push_back(Left{cols, cols[0], 0});
+        const int32_t n = fe.j1, last = cols[n - 1];
+        int32_t k = 0, edge = f + wide;
+        for (int32_t j = 0; j < n;) {
+          const int32_t first = cols[j];
+          for (; first >= edge; edge += wide) ++k;
+          fe.j0 = (int16_t)j;
+          if (last < edge)
+            j = n;
+          else if (last - first == n - 1 - j)  // consecutive columns from here on
+            j += edge - first;
+          else
+            while (cols[j] < edge) ++j;
+          fe.j1 = (int16_t)j;
+          win[k].push_back(fe);
+        }
       }
       int32_t n = 0;
       for (int32_t c0 = 0; c0 < w; c0 += wide) {
-        const int32_t c1 = std::min(w, c0 + wide);
-        const int64_t e0 = (int64_t)P.fan_ent.size();
-        for (int64_t e = G.e0; e < G.e1; ++e) {
-          FanEnt fe = P.fan_ent[e];
-          Left& l = left[e - G.e0];  // the tile's columns from here on lie at c0 or beyond
-          const int32_t end = f + c1;
-          if (l.next >= end) continue;
-          fe.j0 = l.j;
-          int16_t j = l.j + 1;
-          while (j < fe.j1 && l.cols[j] < end) ++j;
-          l.j = j;
-          l.next = j < fe.j1 ? l.cols[j] : INT32_MAX;
-          fe.j1 = j;
-          P.fan_ent.push_back(fe);
-        }
-        const int64_t e1 = (int64_t)P.fan_ent.size();
-        if (e0 == e1) continue;  // no tile has a column there
-        gat.push_back(GatherTask{e0, e1, G.pc, (int16_t)c0, (int16_t)c1});
+        std::vector<FanEnt>& l = win[c0 / wide];
+        if (l.empty()) continue;  // no tile has a column there
+        put(G, l.data(), l.data() + l.size(), c0, std::min(w, c0 + wide));
+        l.clear();
         ++n;
       }
       (o < P.ns ? P.gdiag0[o] : P.tdep0[o - P.ns]) += n - 1;
@@ -928,6 +939,7 @@ void split_gathers(Plan& P, int64_t max_values) {
   P.n_factor_tasks += more;
   P.n_hi_tasks += more;
   P.gat.swap(gat);
+  P.gat_ent.swap(ent);
 }
 
 }  // namespace spchol

@@ -510,3 +510,47 @@ def test_split_gathers_keep_the_order_of_every_entry(name, W, max_values):
         assert got[0] == 0
         np.testing.assert_array_equal(got[1], want[1])
         np.testing.assert_array_equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("name,W,max_values", [("lap3d_12", 64, 1), ("lap3d_12", 20, 300), ("diff3d_9", 16, 64),
+                                               ("lap2d_24", 128, 40), ("lap3d_20", 64, -1), ("lap3d_9", 64, 10**9)])
+def test_split_gather_lists_hold_only_what_the_tasks_add(name, W, max_values):
+    """The lists that the gather tasks index: one task's after another's, with
+    no entry that no task reads; per piece, windows of whole multiples of 8
+    columns whose entries are the unsplit list's, in its order, cut at the
+    windows' edges (found here by a search in the tile's columns)."""
+    A, perm, b = gridgen.workload(name)
+    P, Q = _plan(A, perm, deterministic=2, max_width=W), _plan(A, perm, deterministic=2, max_width=W)
+    Q.split_gathers(max_values)
+    ut = P.get(hp.UTASKS).reshape(-1, 6)
+    fcol, rows, rowoff = P.get(hp.FCOL), P.get(hp.ROWS), P.get(hp.ROWOFF)
+    old, ent0 = P.get(hp.GATHERS).reshape(-1, 5), P.get(hp.GATENT).reshape(-1, 5)
+    assert np.array_equal(ent0[:, :3], P.get(hp.FANENT).reshape(-1, 3))
+    new, ent = Q.get(hp.GATHERS).reshape(-1, 5), Q.get(hp.GATENT).reshape(-1, 5)
+    assert new[0, 0] == 0 and new[-1, 1] == len(ent) and np.array_equal(new[1:, 0], new[:-1, 1])
+    assert np.all(new[:, 0] < new[:, 1])
+    k = 0
+    for e0, e1, pc, c0, c1 in old:
+        listed = ent0[e0:e1]
+        s, t, seg0, seglen = ut[listed[0, 0]][:4]
+        f, w = fcol[t], fcol[t + 1] - fcol[t]
+        assert (c0, c1) == (0, w)
+        k0 = k
+        while k < len(new) and new[k, 2] == pc:
+            k += 1
+        windows = new[k0:k]
+        assert np.all(windows[1:, 3] >= windows[:-1, 4]) and windows[-1, 4] <= w
+        assert np.all(windows[:, 3] % 8 == 0) and np.all((windows[:, 4] % 8 == 0) | (windows[:, 4] == w))
+        columns = 0
+        for a, e, _, lo, hi in windows:
+            want = []
+            for u, i0, i1, _, _ in listed:
+                s, t, seg0, seglen = ut[u][:4]
+                cols = rows[rowoff[s] + seg0:rowoff[s] + seg0 + seglen] - f
+                j0, j1 = np.searchsorted(cols, [lo, hi])
+                if j0 < j1:
+                    want.append((u, i0, i1, j0, j1))
+            assert np.array_equal(ent[a:e], want)
+            columns += sum(q[4] - q[3] for q in want)
+        assert columns == ut[listed[:, 0], 3].sum()
+    assert k == len(new)
