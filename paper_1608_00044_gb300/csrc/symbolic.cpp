@@ -387,6 +387,10 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
   P.trsm_sn.clear();
   P.ut.clear();
   P.n_rel = 0;
+  // The rows below each panel's diagonal block by target panel: where each
+  // target's end, one panel's after another's (found once, walked three times).
+  std::vector<int32_t> seg_end;
+  seg_end.reserve(4 * (size_t)ns);
   // ---- rows per update and panel-solve tile, level by level (PlanParams::level_tiles)
   std::vector<int32_t> upd_rows, solve_rows;
   {
@@ -402,7 +406,9 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
       for (int q = 0; q < 2; ++q) t[q] += (r - w + tr[q] - 1) / tr[q];
       for (int32_t a = w; a < r;) {
         for (int q = 0; q < 2; ++q) u[q] += (r - a + ur[q] - 1) / ur[q];
-        a = (int32_t)(std::lower_bound(R + a, R + r, P.fcol[P.snode_of[R[a]] + 1]) - R);
+        const int32_t end = P.fcol[P.snode_of[R[a]] + 1];
+        while (a < r && R[a] < end) ++a;
+        seg_end.push_back(a);
       }
     }
     // FP64 tiles: more of them per CTA on the larger problems (see there)
@@ -428,22 +434,17 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     // the tile count first (the same walk), so that the tile list is built in
     // place: millions of tiles on the large grids
     int64_t nt = 0, ntr = 0;
+    const int32_t* e = seg_end.data();
     for (int32_t s = 0; s < ns; ++s) {
       const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
       const int TU = update_rows(s), TR = trsm_rows(s);
       ntr += (r - w + TR - 1) / TR;
-      const int32_t* R = P.rows.data() + P.rowoff[s];
-      for (int32_t a = w; a < r;) {
-        const int32_t t = P.snode_of[R[a]];
-        int32_t e = a;
-        while (e < r && R[e] < P.fcol[t + 1]) ++e;
-        nt += (r - a + TU - 1) / TU;
-        a = e;
-      }
+      for (int32_t a = w; a < r; a = *e++) nt += (r - a + TU - 1) / TU;
     }
     P.ut.reserve((size_t)nt);
     P.trsm_sn.reserve((size_t)ntr);
   }
+  const int32_t* seg = seg_end.data();
   for (int32_t s = 0; s < ns; ++s) {
     const int32_t w = P.fcol[s + 1] - P.fcol[s], r = P.nrows[s];
     const int32_t nb = r - w;
@@ -457,9 +458,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
     const int32_t* R = P.rows.data() + P.rowoff[s];
     int32_t a = w;
     while (a < r) {
-      int32_t t = P.snode_of[R[a]];
-      int32_t e = a;
-      while (e < r && R[e] < P.fcol[t + 1]) ++e;
+      const int32_t t = P.snode_of[R[a]], e = *seg++;
       for (int32_t r0 = a; r0 < r; r0 += TU) {
         const int32_t len = std::min(TU, r - r0);
         P.ut.push_back(UTask{s, t, a, e - a, r0, len, P.n_rel});
