@@ -1212,6 +1212,39 @@ int solve_refined(spchol_handle_t h, int nrhs, cudaStream_t st) {
   return rc;
 }
 
+// One analysis with the options as they are.
+int analyze_impl(int64_t n, const int64_t* colptr, const int32_t* rowind, const int64_t* perm, const spchol_options& o,
+                 std::chrono::steady_clock::time_point t0, spchol_handle_t* out) {
+  spchol_handle_t h = new (std::nothrow) spchol_handle_s();
+  if (!h) return SPCHOL_ENOMEM;
+  clear_stale_error();
+  h->opt = o;
+  h->fp32 = (o.precision == SPCHOL_FP32 || o.precision == SPCHOL_TF32 || o.precision == SPCHOL_TF32X3);
+  if (cudaGetDevice(&h->device) != cudaSuccess) {
+    delete h;
+    return SPCHOL_ECUDA;
+  }
+  PlanError err;
+  int rc = build_plan(n, colptr, rowind, perm, params_from(o), h->plan, err);
+  if (rc == 0 && h->fp32) {
+    h->a_row.resize(h->plan.nnz_a);
+    h->a_col.resize(h->plan.nnz_a);
+    for (int64_t j = 0; j < n; ++j)
+      for (int64_t p = colptr[j]; p < colptr[j + 1]; ++p) {
+        h->a_row[p] = rowind[p];
+        h->a_col[p] = (int32_t)j;
+      }
+  }
+  if (rc == 0 && o.fault_inject == 1 && h->plan.ns > 0) h->plan.dep_f[h->plan.ns - 1] += 1;
+  if (rc == 0) rc = finish_analyze(h, t0);
+  if (rc != 0) {
+    spchol_destroy(h);
+    return rc;
+  }
+  *out = h;
+  return 0;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1251,34 +1284,13 @@ int spchol_analyze(int64_t n, const int64_t* colptr, const int32_t* rowind, cons
   } else {
     spchol::default_options(&o);
   }
-  spchol_handle_t h = new (std::nothrow) spchol_handle_s();
-  if (!h) return SPCHOL_ENOMEM;
-  clear_stale_error();
-  h->opt = o;
-  h->fp32 = (o.precision == SPCHOL_FP32 || o.precision == SPCHOL_TF32 || o.precision == SPCHOL_TF32X3);
-  if (cudaGetDevice(&h->device) != cudaSuccess) {
-    delete h;
-    return SPCHOL_ECUDA;
+  int rc = analyze_impl(n, colptr, rowind, perm, o, t0, out);
+  if (rc == SPCHOL_ENOMEM && o.solve_w_depth == 0 && !o.deterministic) {
+    // the default depth's W is no reason to refuse a matrix whose factor fits
+    o.solve_w_depth = kWDepthLow;
+    rc = analyze_impl(n, colptr, rowind, perm, o, t0, out);
   }
-  PlanError err;
-  int rc = build_plan(n, colptr, rowind, perm, params_from(o), h->plan, err);
-  if (rc == 0 && h->fp32) {
-    h->a_row.resize(h->plan.nnz_a);
-    h->a_col.resize(h->plan.nnz_a);
-    for (int64_t j = 0; j < n; ++j)
-      for (int64_t p = colptr[j]; p < colptr[j + 1]; ++p) {
-        h->a_row[p] = rowind[p];
-        h->a_col[p] = (int32_t)j;
-      }
-  }
-  if (rc == 0 && o.fault_inject == 1 && h->plan.ns > 0) h->plan.dep_f[h->plan.ns - 1] += 1;
-  if (rc == 0) rc = finish_analyze(h, t0);
-  if (rc != 0) {
-    spchol_destroy(h);
-    return rc;
-  }
-  *out = h;
-  return 0;
+  return rc;
 }
 
 int spchol_factorize(spchol_handle_t h, const double* values, void* stream) {

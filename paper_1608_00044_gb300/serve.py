@@ -116,13 +116,17 @@ class Server:
                 r.busy += 1
                 r.last_use = time.perf_counter()
                 return r, False
-        h = spchol.analyze(A.n, A.colptr, A.rowind, perm, spchol.default_options(**self.opt_kw))
         # the factor plus the solve workspace (Y and B; X and R too with refinement)
         # for the most right-hand sides any request may bring
         nrhs = max(self.max_nrhs, req.B.shape[1], 1)
-        fp = spchol.stats(h)["footprint_bytes"] + (4 if self.fp32 else 2) * A.n * nrhs * 8
-        if fp > self.budget:  # could never fit, even with every other factor evicted
+        for depth in (0, 32):  # a factor that does not fit with the default's W panels gets fewer
+            h = spchol.analyze(A.n, A.colptr, A.rowind, perm,
+                               spchol.default_options(**self.opt_kw, solve_w_depth=depth))
+            fp = spchol.stats(h)["footprint_bytes"] + (4 if self.fp32 else 2) * A.n * nrhs * 8
+            if fp <= self.budget:
+                break
             spchol.destroy(h)
+        else:  # could never fit, even with every other factor evicted
             with self.mem_cv:
                 self.rejected += 1
             return None, False

@@ -292,3 +292,58 @@ def test_torch_allocator_batch_handle():
     for a_, b_ in zip(*Xs_all):
         assert np.array_equal(a_, b_)
     assert alloc.held_bytes() == held0
+
+
+def test_memory_for_fewer_w_panels_is_enough():
+    # The default keeps W panels for 64 levels, 5.7 MB more than 32 levels do on
+    # a 24^3 Laplacian: an allocator that holds the smaller footprint and
+    # half of the difference gets a handle (with 32 levels), one that holds
+    # less than that ENOMEM, and a depth that the caller gives is not lowered.
+    import ctypes
+
+    A, perm, _ = gridgen.workload("lap3d_24")
+    fp = {}
+    for depth in (0, 32):
+        h = spchol.analyze(A.n, A.colptr, A.rowind, perm, spchol.default_options(solve_w_depth=depth))
+        fp[depth] = spchol.stats(h)["footprint_bytes"]
+        spchol.destroy(h)
+    assert fp[0] > fp[32] + (1 << 20)
+    base = spchol.torch_allocator()
+    state = {"limit": 0, "held": 0}
+
+    def alloc(nbytes, stream, ctx):
+        if state["held"] + nbytes > state["limit"]:
+            return None
+        p = base._alloc(nbytes, stream, ctx)
+        if p:
+            state["held"] += nbytes
+        return p
+
+    def free(ptr, nbytes, stream, ctx):
+        state["held"] -= nbytes
+        base._free(ptr, nbytes, stream, ctx)
+
+    acb, fcb = spchol.DEV_ALLOC_FN(alloc), spchol.DEV_FREE_FN(free)
+
+    def opts(**kw):
+        o = spchol.default_options(**kw)
+        o.dev_alloc = ctypes.cast(acb, ctypes.c_void_p).value
+        o.dev_free = ctypes.cast(fcb, ctypes.c_void_p).value
+        return o
+
+    between = (fp[0] + fp[32]) // 2
+    for limit, depth, ok in ((between, 0, True), (between, 64, False), (fp[32] // 2, 0, False)):
+        state["limit"] = limit
+        if not ok:
+            with pytest.raises(spchol.SpcholError) as e:
+                spchol.analyze(A.n, A.colptr, A.rowind, perm, opts(solve_w_depth=depth))
+            assert e.value.code == spchol.ENOMEM and state["held"] == 0
+            continue
+        h = spchol.analyze(A.n, A.colptr, A.rowind, perm, opts(solve_w_depth=depth))
+        assert spchol.stats(h)["footprint_bytes"] == fp[32]
+        state["limit"] = 1 << 40
+        assert spchol.factorize(h, _dev(A.values)) == 0
+        B = gridgen.rhs_uniform(A.n, 2, seed=5)
+        assert oracle.berr(A, _solve_dev(h, B), B) <= BERR_FP64
+        spchol.destroy(h)
+        assert state["held"] == 0

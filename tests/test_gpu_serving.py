@@ -116,3 +116,25 @@ def test_repeat_solve_with_more_rhs_stays_inside_the_budget():
         assert r.footprint >= st["footprint_bytes"] + 2 * st["n"] * 16 * 8
     assert s.peak_used <= s.budget
     s.close()
+
+
+def test_budget_for_fewer_w_panels_serves_the_request():
+    # A request whose factor fits the budget with 32 levels of W panels, but not
+    # with the default's 64, is served (the default alone refused it).
+    import gridgen
+
+    A, perm, b = gridgen.workload("lap3d_24")
+    fp = {}
+    for depth in (0, 32):
+        h = spchol.analyze(A.n, A.colptr, A.rowind, perm, spchol.default_options(solve_w_depth=depth))
+        fp[depth] = spchol.stats(h)["footprint_bytes"] + 2 * A.n * 16 * 8
+        spchol.destroy(h)
+    assert fp[0] > fp[32]
+    for budget, rc in (((fp[0] + fp[32]) // 2, 0), (fp[32] - 1, spchol.ENOMEM)):
+        q = serve.Request(rid=0, arrival=0.0, key="k", vkey="v", make=lambda: (A, perm), B=b.copy(order="F"))
+        s = serve.Server(slots=1, budget_bytes=budget)
+        s.run([q])
+        assert q.rc == rc and s.rejected == (rc != 0) and s.peak_used <= budget
+        if rc == 0:
+            assert oracle.berr(A, q.X, b) <= 1e-13
+        s.close()
