@@ -879,8 +879,11 @@ __device__ void bwd_tile_fma(const SolveArgs& a, const T* P, int ld, int row0, i
   const int tid = threadIdx.x;
   const int nchunk = (cnt + kTileCH - 1) / kTileCH;
   const int xi = tid % kTileCH, xr = tid / kTileCH;    // the x entry this thread loads (256 = 8 x 32)
-  for (int r0 = 0; r0 < a.nrhs; r0 += kSolveNRC) {
-    const int nrc = min(kSolveNRC, a.nrhs - r0);
+  // a thread has two outputs, which panels wider than 64 reach with fewer right-hand sides a pass
+  static_assert(64 * kSolveNRC <= 2 * kSolveThreads, "two outputs a thread");
+  const int most = w <= 64 ? kSolveNRC : 2 * kSolveThreads / w;
+  for (int r0 = 0; r0 < a.nrhs; r0 += most) {
+    const int nrc = min(most, a.nrhs - r0);
     const int O = w * nrc;
     const int RG = O <= 64 ? 4 : O <= 128 ? 2 : 1;
     const int per = blockDim.x / RG, rg = tid / per, u = tid - rg * per;

@@ -1018,3 +1018,29 @@ def test_warp_subtree_solves_of_many_right_hand_sides(precision, bar, nrhs, widt
     X, B = np.concatenate(Xs), np.concatenate(Bs)
     for r in range(nrhs):
         assert oracle.berr(A, np.asfortranarray(X[:, r:r + 1]), np.asfortranarray(B[:, r:r + 1])) <= bar
+
+
+@pytest.mark.parametrize("W,nrhs", [(64, 8), (65, 7), (65, 8), (73, 7), (74, 7), (85, 6), (102, 5), (103, 5), (96, 11),
+                                    (128, 4), (128, 5), (128, 8), (128, 13)])
+@pytest.mark.parametrize("precision,deterministic", [("FP64", 0), ("FP64", 2), ("FP32", 0)])
+def test_solves_of_panels_wider_than_64_with_several_right_hand_sides(W, nrhs, precision, deterministic):
+    # A backward tile of a panel of w columns has w nrhs outputs a pass, two a
+    # thread: 512 at most, on either side of which these lie.  Every
+    # right-hand side's backward error, and in FP64 the
+    # solution against the oracle's.
+    A, perm, _ = gridgen.workload("lap3d_12")
+    B = gridgen.rhs_uniform(A.n, nrhs, seed=W)
+    s = spchol.SparseCholesky(A.n, A.colptr, A.rowind, perm, max_width=W, relax_zeros=32, deterministic=deterministic,
+                              precision=getattr(spchol, precision))
+    assert s.stats()["max_width"] == W
+    assert s.factorize(A.values) == 0
+    X = s.solve(B.copy(order="F"))
+    s.close()
+    for r in range(nrhs):
+        berr = oracle.berr(A, np.asfortranarray(X[:, r:r + 1]), np.asfortranarray(B[:, r:r + 1]))
+        assert berr <= (BERR_FP64 if precision == "FP64" else 1e-12), (r, berr)
+    if precision == "FP64":
+        f = oracle.OracleFactor.from_csc(A, perm)
+        assert f.factor() == 0
+        Xo = f.solve(B)
+        assert np.abs(X - Xo).max() <= 1e-10 * np.abs(Xo).max()
