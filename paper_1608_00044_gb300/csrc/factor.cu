@@ -25,7 +25,6 @@ namespace spchol {
 
 namespace {
 
-constexpr int kTrsmJB = 8;     // wide panels: columns solved together per row (independent FMA chains)
 constexpr int kTrsmMaxW = 64;  // panels up to this width take the register-resident panel solve
 
 struct FactorShared {
@@ -303,14 +302,14 @@ __device__ void invert_l11(double* sm, const double* xd, int w, double* __restri
   }
 }
 
-// L21 = A21 L11^{-T} for rows row0 .. row0 + cnt - 1 of a panel at most
-// kTrsmMaxW wide, row by row: forward substitution along each row with the
+// L21 = A21 L11^{-T} for rows row0 .. row0 + cnt - 1 of a panel at most 8 NC
+// wide, row by row: forward substitution along each row with the
 // columns in registers.  Warp q takes 4-row strips 4 (q + 8 v); lane (lr, lc)
 // holds row lr of the strip at columns lc + 8 cc.  Step c: the lane holding
 // column c scales it by rinv[c] = 1 / l_cc, the value is broadcast within the 8
 // lanes of the row, and every later column subtracts it times l_qc = Ls[q + ldl
 // c] (read past row w only for columns that are not stored).
-template <typename T>
+template <int NC, typename T>
 __device__ __forceinline__ void trsm_strips(T* P, int ld, int row0, int cnt, int w, const T* Ls, int ldl,
                                             const T* rinv) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane >> 3, lc = lane & 7;
@@ -319,14 +318,14 @@ __device__ __forceinline__ void trsm_strips(T* P, int ld, int row0, int cnt, int
     const int rloc = 4 * st + lr;
     const bool rv = rloc < cnt;
     T* Pi = P + row0 + rloc;
-    T x[8];
+    T x[NC];
 #pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
+    for (int cc = 0; cc < NC; ++cc) {
       const int c = lc + 8 * cc;
       x[cc] = (rv && c < w) ? ldcg(Pi + (size_t)c * ld) : T(0);
     }
 #pragma unroll
-    for (int cbk = 0; cbk < 8; ++cbk) {
+    for (int cbk = 0; cbk < NC; ++cbk) {
       if (8 * cbk >= w) break;
       for (int c8 = 0; c8 < 8; ++c8) {
         const int c = 8 * cbk + c8;
@@ -336,14 +335,14 @@ __device__ __forceinline__ void trsm_strips(T* P, int ld, int row0, int cnt, int
         const T* Lc = Ls + ldl * c;
         if (lc > c8) x[cbk] -= xc * Lc[lc + 8 * cbk];
 #pragma unroll
-        for (int cc = cbk + 1; cc < 8; ++cc) {
+        for (int cc = cbk + 1; cc < NC; ++cc) {
           if (8 * cc >= w) break;
           x[cc] -= xc * Lc[lc + 8 * cc];
         }
       }
     }
 #pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
+    for (int cc = 0; cc < NC; ++cc) {
       const int c = lc + 8 * cc;
       if (rv && c < w) Pi[(size_t)c * ld] = x[cc];
     }
@@ -478,13 +477,13 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
     if (FUSE && fuse) {  // the rows below, with L11 from shared memory (in the panel's type)
       const int nb = a.pv.nrows[s] - w;
       if constexpr (sizeof(T) == 8) {
-        trsm_strips<T>(P, ld, w, nb, w, sm, w, xd);
+        trsm_strips<kFuseWidth / 8>(P, ld, w, nb, w, sm, w, xd);
       } else {
         T *Lf = reinterpret_cast<T*>(xd + w), *rf = Lf + w * w;
         for (int idx = tid; idx < w * w; idx += blockDim.x) Lf[idx] = (T)sm[idx];
         for (int j = tid; j < w; j += blockDim.x) rf[j] = (T)xd[j];
         __syncthreads();
-        trsm_strips<T>(P, ld, w, nb, w, Lf, w, rf);
+        trsm_strips<kFuseWidth / 8>(P, ld, w, nb, w, Lf, w, rf);
       }
     }
     for (int j = warp; j < w; j += kFactorThreads / 32)
@@ -589,6 +588,25 @@ __device__ void slice_row(const double* Pi, int w, int ld, int kpad, int nb, int
 // ---------------------------------------------------------------- TRSM(s, k)
 // Arithmetic in the panel's type: FP64 panels solve in FP64, FP32 panels (the
 // mixed-precision modes) in FP32.
+// Panels wider than kTrsmMaxW (CUDA-core tiles only): the same rows, 16 columns
+// a lane, with the whole of L11 in shared memory.  What bounds it is the chain
+// of w steps.  (A thread a row, its solved columns read back from L2 in blocks
+// of 8, kept 16 of the CTA's threads busy with a 16-row tile, each waiting for
+// one trip after another: 602 us a tile of a 128-column panel, FP32 470, now 73
+// and 59.  Factorization of a full matrix of order 1500 with max_width 128: 9.9 ->
+// 4.05 ms, FP32 7.9 -> 3.3; 31^3 Laplacian with relax_zeros 32: 20.5 -> 10.0.)
+template <typename T>
+__device__ __forceinline__ void trsm_wide(T* P, int ld, int row0, int cnt, int w, T* Ls, const double* Xd) {
+  T* rinv = Ls + w * w;
+  for (int idx = threadIdx.x; idx < w * w; idx += kFactorThreads) {
+    const int i = idx % w, j = idx / w;
+    Ls[idx] = i > j ? ldcg(P + i + (size_t)j * ld) : T(0);
+  }
+  for (int c = threadIdx.x; c < w; c += kFactorThreads) rinv[c] = (T)ldcg(Xd + c * (w + 1));
+  __syncthreads();
+  trsm_strips<16>(P, ld, row0, cnt, w, Ls, w, rinv);
+}
+
 template <typename T, int MODE>
 __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, FactorShared& sh, bool skip,
                           bool release = true) {
@@ -611,7 +629,7 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
     const double* Xd = a.inv + a.invoff[s];
     for (int c = tid; c < w; c += nt) rinv[c] = (ct)ldcg(Xd + c * (w + 1));  // written by the diagonal task
     __syncthreads();
-    trsm_strips<T>(P, ld, row0, cnt, w, Ls, kTrsmMaxW, rinv);
+    trsm_strips<kTrsmMaxW / 8>(P, ld, row0, cnt, w, Ls, kTrsmMaxW, rinv);
     if constexpr (sizeof(T) == 8 && MODE == 3) {
       if (w >= a.tc_min_width) {
         __syncthreads();  // the tile's rows are written (visible to this CTA through L2)
@@ -622,48 +640,8 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
       }
     }
   } else if (!skip) {
-    // Panels wider than kTrsmMaxW: one thread per row, columns in blocks.
-    if constexpr (sizeof(ct) == 8) {
-      stage_lower<true>(P, w, ld, reinterpret_cast<double*>(sm));
-    } else {
-      for (int idx = tid; idx < w * w; idx += nt) {
-        const int i = idx % w, j = idx / w;
-        sm[idx] = (i >= j) ? (ct)ldcg(P + i + (size_t)j * ld) : ct(0);
-      }
-    }
-    __syncthreads();
-    for (int rr = tid; rr < cnt; rr += nt) {
-      T* Pi = P + row0 + rr;
-      for (int jb = 0; jb < w; jb += kTrsmJB) {
-        const int nb = min(kTrsmJB, w - jb);
-        ct x[kTrsmJB];
-#pragma unroll
-        for (int c = 0; c < kTrsmJB; ++c) x[c] = (c < nb) ? (ct)ldcg(Pi + (size_t)(jb + c) * ld) : ct(0);
-        for (int kk = 0; kk < jb; ++kk) {
-          const ct xk = (ct)ldcg(Pi + (size_t)kk * ld);
-          const ct* Lk = sm + kk * w + jb;  // L[jb + c][kk]
-#pragma unroll
-          for (int c = 0; c < kTrsmJB; ++c)
-            if (c < nb) x[c] -= xk * Lk[c];
-        }
-#pragma unroll
-        for (int c = 0; c < kTrsmJB; ++c) {
-          if (c < nb) {
-#pragma unroll
-            for (int c2 = 0; c2 < c; ++c2) x[c] -= x[c2] * sm[(jb + c) + (jb + c2) * w];
-            x[c] = x[c] / sm[(jb + c) + (jb + c) * w];
-            Pi[(size_t)(jb + c) * ld] = (T)x[c];
-          }
-        }
-      }
-      if constexpr (sizeof(T) == 8 && MODE == 3) {
-        if (w >= a.tc_min_width) {
-          const int kpad = (w + 15) & ~15, nbel = r - w, ib = row0 + rr - w;
-          slice_row(reinterpret_cast<const double*>(Pi), w, ld, kpad, nbel, ib, a.slices + a.sliceoff[s],
-                    a.rexp + a.pv.rowoff[s] + row0 + rr);
-        }
-      }
-    }
+    // (the tensor-core modes have no such panels: options_valid)
+    if constexpr (MODE == 0) trsm_wide<T>(P, ld, row0, cnt, w, sm, a.inv + a.invoff[s]);
   }
   publish_cta_writes();
   if (!release) return;  // inside a subtree task: no counters, the same CTA goes on

@@ -1044,3 +1044,31 @@ def test_solves_of_panels_wider_than_64_with_several_right_hand_sides(W, nrhs, p
         assert f.factor() == 0
         Xo = f.solve(B)
         assert np.abs(X - Xo).max() <= 1e-10 * np.abs(Xo).max()
+
+
+@pytest.mark.parametrize("precision", ["FP64", "FP32"])
+@pytest.mark.parametrize("w,m", [(64, 7), (65, 1), (66, 5), (71, 33), (72, 64), (73, 17), (96, 100), (127, 70), (128, 131)])
+def test_panels_wider_than_64_solve_their_rows(w, m, precision):
+    # A full matrix of order w + m cut at w columns: the first panel's solve of
+    # its m rows below holds 16 columns a lane past 64 (tiles of 64, 32 and 16
+    # rows, strips with 1 to 4 of them).  Its condition number is below 8, so L
+    # is within 8 n roundings of the dense factor's, in FP32 the rows'.
+    n = w + m
+    rng = np.random.default_rng(1000 * w + m)
+    M = rng.uniform(-1.0, 1.0, (n, n))
+    A = np.eye(n) + (M + M.T) / (4.0 * n)
+    cp = np.concatenate([[0], np.cumsum(np.arange(n, 0, -1))]).astype(np.int64)
+    ri = np.concatenate([np.arange(j, n) for j in range(n)]).astype(np.int32)
+    s = spchol.SparseCholesky(n, cp, ri, max_width=w, precision=getattr(spchol, precision))
+    assert s.factorize(np.concatenate([A[j:, j] for j in range(n)])) == 0
+    Lp, Li, Lx, perm = s.export_factor()
+    L = np.zeros((n, n))
+    for j in range(n):
+        L[Li[Lp[j]:Lp[j + 1]], j] = Lx[Lp[j]:Lp[j + 1]]
+    want = np.linalg.cholesky(A[np.ix_(perm, perm)])
+    eps = 2.0 ** -53 if precision == "FP64" else 2.0 ** -24
+    assert np.abs(L - want).max() <= 8 * 8 * n * eps * np.abs(want).max()
+    b = rng.uniform(-1.0, 1.0, (n, 2))
+    X = s.solve(b.copy(order="F"))
+    s.close()
+    assert np.abs(X - np.linalg.solve(A, b)).max() <= (64 * n * 2.0 ** -53 if precision == "FP64" else 1e-10)
