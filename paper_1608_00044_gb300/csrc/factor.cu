@@ -153,7 +153,7 @@ __device__ __forceinline__ void pivot_load(const double* sm, int w, int c, int i
 // columns after it are not meaningful and are not used.
 template <bool MAIN>
 __device__ __forceinline__ void pivot_pair(const FactorArgs& a, double* sm, double* xd, int w, int c, int f,
-                                           bool both) {
+                                           bool both, FactorShared& sh) {
   const int lane = threadIdx.x & 31;
   const bool two = c + 1 < w;
   constexpr int kL = MAIN ? 0 : 30;  // the lanes that hold rows c and c + 1
@@ -179,8 +179,11 @@ __device__ __forceinline__ void pivot_pair(const FactorArgs& a, double* sm, doub
     if (lane == 0) {
       xd[c] = r2;
       if (two) xd[c + 1] = r3;
-      if (!pivot_positive(d2)) atomicMin(&a.ctrl[kInfo], f + c + 1);
-      if (!pivot_positive(d3)) atomicMin(&a.ctrl[kInfo], f + c + 2);
+      const bool bad2 = !pivot_positive(d2);
+      if (bad2 || !pivot_positive(d3)) {
+        atomicMin(&a.ctrl[kInfo], f + c + (bad2 ? 1 : 2));
+        sh.flag = 1;
+      }
     }
   }
   double* c2 = sm + c * w;
@@ -247,6 +250,7 @@ __device__ void invert_l11(double* sm, const double* xd, int w, double* __restri
       X[i + (size_t)(r0 + lc + 4) * w] = x1;
     }
   }
+  if (nb == 1) return;
   __syncthreads();
   // G_b for all block rows: group t of 4 columns of block row b (2 b of them)
   for (int g = warp; g < nb * (nb - 1); g += kFactorThreads / 32) {
@@ -438,6 +442,8 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   const bool fuse = FUSE && fused_panel(a, s, w);
   if (!skip) {
     stage_lower<true>(P, w, ld, sm);  // lower triangle; zeros above (used below for L11^{-1})
+    if (tid == 0) sh.flag = 0;  // 1: a failed pivot, whose columns are not used (a word of the CTA's own: the
+                                // status word is a trip to L2 ahead of the release)
     const int uw = warp == 3 ? kUpdWarps - 1 : warp > 3 ? warp - 1 : warp;  // number among the update warps
     const int ut = uw * 32 + lane;
     constexpr int kStep = kUpdWarps * 32;
@@ -453,9 +459,9 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
     __syncthreads();
     for (int c = 0; c < w; c += 2) {
       if (warp == kPivotWarp) {
-        pivot_pair<true>(a, sm, xd, w, c, f, w - c > 32);
+        pivot_pair<true>(a, sm, xd, w, c, f, w - c > 32, sh);
       } else if (warp == kPivotWarp - 1) {
-        if (w - c > 32) pivot_pair<false>(a, sm, xd, w, c, f, true);
+        if (w - c > 32) pivot_pair<false>(a, sm, xd, w, c, f, true, sh);
       } else if (c > 0) {
         const int m = w - 2 - c;  // columns c + 2 .. w - 1
         const int np = m > 0 ? m * (m + 1) / 2 : 0;
@@ -472,8 +478,6 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
       }
       __syncthreads();
     }
-    // a failed pivot, of this block or of any other: its columns are not used
-    if (tid == 0) sh.flag = ld_relaxed(&a.ctrl[kInfo]) != INT_MAX;
     if (FUSE && fuse) {  // the rows below, with L11 from shared memory (in the panel's type)
       const int nb = a.pv.nrows[s] - w;
       if constexpr (sizeof(T) == 8) {
