@@ -176,6 +176,9 @@ __device__ __forceinline__ void pivot_pair(const FactorArgs& a, double* sm, doub
   }
   if (MAIN) {
     if (both) asm volatile("bar.sync 1, 64;" ::: "memory");
+    // an infinite pivot's root is infinite (r is 0, and inf * 0 no number)
+    if (lane == 0 && __double2hiint(d2) == 0x7ff00000) x2 = d2;
+    if (lane == 1 && __double2hiint(d3) == 0x7ff00000) x3 = d3;
     if (lane == 0) {
       xd[c] = r2;
       if (two) xd[c + 1] = r3;
@@ -1713,6 +1716,7 @@ __device__ __forceinline__ bool warp_factor(double* A, int la, int R, int w, dou
     const double y = pivot_rsqrt(d);
     if (lane == 0) xd[j] = y;
     for (int i = j + lane; i < R; i += 32) cj[i] *= y;
+    if (lane == 0 && __double2hiint(d) == 0x7ff00000) cj[j] = d;  // (y is 0, and inf * 0 no number)
     __syncwarp();
     const int m = R - j - 1, nc = w - j - 1;
     if (nc > 0) {

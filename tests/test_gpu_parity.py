@@ -1072,3 +1072,59 @@ def test_panels_wider_than_64_solve_their_rows(w, m, precision):
     X = s.solve(b.copy(order="F"))
     s.close()
     assert np.abs(X - np.linalg.solve(A, b)).max() <= (64 * n * 2.0 ** -53 if precision == "FP64" else 1e-10)
+
+
+@pytest.mark.parametrize("w", [1, 2, 3, 5, 33, 40])
+def test_infinite_pivots(w):
+    # A dense block with one infinite diagonal entry: its column of L is
+    # infinite on the diagonal and zero below, its unknown zero, and the others
+    # those of the system without it.
+    rng = np.random.default_rng(w)
+    M = rng.uniform(-1.0, 1.0, (w, w))
+    A = np.eye(w) + (M + M.T) / (4.0 * max(w, 2))
+    k = w // 2
+    A[k, k] = np.inf
+    rest = np.arange(w) != k
+    b = rng.uniform(-1.0, 1.0, (w, 1))
+    cp = np.concatenate([[0], np.cumsum(np.arange(w, 0, -1))]).astype(np.int64)
+    ri = np.concatenate([np.arange(j, w) for j in range(w)]).astype(np.int32)
+    vals = np.concatenate([A[j:, j] for j in range(w)])
+    s = spchol.SparseCholesky(w, cp, ri, max_width=64)
+    assert s.factorize(vals) == 0
+    Lp, Li, Lx, perm = s.export_factor()
+    L = np.zeros((w, w))
+    for j in range(w):
+        L[Li[Lp[j]:Lp[j + 1]], j] = Lx[Lp[j]:Lp[j + 1]]
+    kk = int(np.flatnonzero(perm == k)[0])
+    assert L[kk, kk] == np.inf and np.all(L[kk + 1:, kk] == 0.0)
+    X = s.solve(b.copy(order="F"))
+    s.close()
+    assert X[k, 0] == 0.0
+    if w > 1:
+        want = np.linalg.solve(A[np.ix_(rest, rest)], b[rest])
+        assert np.abs(X[rest] - want).max() <= 64 * w * 2.0 ** -53 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("precision", ["FP64", "FP32"])
+def test_infinite_pivots_in_warp_subtrees(precision):
+    # The same in a batch whose panels run on single warps: infinite diagonals of
+    # L there and nowhere else, no NaN, and zero for those unknowns.
+    sides = np.random.default_rng(3).integers(20, 60, 64)
+    mats = [gridgen.diffusion_2d_5pt(int(q), seed=i) for i, q in enumerate(sides)]
+    h = spchol.batch_analyze([M.n for M in mats], [M.colptr for M in mats], [M.rowind for M in mats],
+                             [gridgen.geometric_nd(M.dims) for M in mats],
+                             spchol.default_options(max_width=32, relax_zeros=16, tile_rows=32,
+                                                    precision=getattr(spchol, precision)))
+    assert spchol.stats(h)["n_warp_subtrees"] == spchol.stats(h)["n_subtrees"] > 0
+    vals = [M.values.copy() for M in mats]
+    infinite = [(t, c) for t in (3, 10, 41) for c in (0, mats[t].n // 3, mats[t].n - 1)]
+    for t, c in infinite:
+        vals[t][mats[t].colptr[c]] = np.inf
+    assert spchol.batch_factorize(h, vals) == 0
+    Lp, Li, Lx, perm = spchol.export_factor(h)
+    assert not np.isnan(Lx).any() and np.isinf(Lx).sum() == len(infinite) and np.isinf(Lx[Lp[:-1]]).sum() == len(infinite)
+    if precision == "FP64":  # (with refinement the residual is not finite)
+        X = [np.ones((M.n, 1), order="F") for M in mats]
+        spchol.batch_solve(h, X, [M.n for M in mats], [1] * len(mats))
+        assert all(np.isfinite(x).all() for x in X) and all(X[t][c, 0] == 0.0 for t, c in infinite)
+    spchol.destroy(h)
