@@ -182,3 +182,33 @@ def test_fp32_panels_of_every_scale(precision, exponent):
         assert oracle.berr(M, X[name], b) <= 1e-12
         s.close()
     assert np.abs(X["scaled"] * 2.0 ** exponent - X["plain"]).max() <= 1e-8 * np.abs(X["plain"]).max()
+
+
+@pytest.mark.parametrize("precision", ["FP32", "TF32X3"])
+@pytest.mark.parametrize("depth", [-1, 0])
+def test_subnormal_entries_of_fp32_panels_count(precision, depth):
+    # The solves widen FP32 entries of L (and of W) to FP64: normal numbers and
+    # zeros by their bits, subnormals by the conversion.  An arrow whose first
+    # column of L is s = k 2^-149, at most the first normals, with pivots
+    # 2^-100 below: the trailing updates s_i s_j vanish, and with panels of one
+    # column every product s y is a panel entry's.  No refinement (ir_tol 1), so
+    # the first solve's result shows: b = e_0 gives x_i = -2^100 s_i, and b_i = 1
+    # gives x_0 = -2^100 sum s, exactly.
+    k = np.array([0, 1, 2, 3, -1, 2 ** 22 - 1, 2 ** 22, -(2 ** 22) - 1, 2 ** 23 - 1, 2 ** 23, 2 ** 23 + 1, -(2 ** 24)])
+    s_ = k * 2.0 ** -149
+    n = 1 + len(k)
+    cp = np.concatenate([[0, n], n + 1 + np.arange(n - 1)]).astype(np.int64)
+    ri = np.concatenate([np.arange(n), np.arange(1, n)]).astype(np.int32)
+    vals = np.concatenate([[1.0], s_, np.full(n - 1, 2.0 ** -100)])
+    s = spchol.SparseCholesky(n, cp, ri, max_width=1, relax_zeros=0, precision=getattr(spchol, precision), ir_tol=1.0,
+                              solve_w_depth=depth)
+    assert s.factorize(vals) == 0
+    Lp, Li, Lx, perm = s.export_factor()
+    assert perm[0] == 0 and np.array_equal(Lx[1:Lp[1]], s_[perm[Li[1:Lp[1]]] - 1])
+    b = np.zeros((n, 2), order="F")
+    b[0, 0] = 1.0
+    b[1:, 1] = 1.0
+    X = s.solve(b)
+    s.close()
+    assert np.array_equal(X[1:, 0], -s_ * 2.0 ** 100)
+    assert X[0, 1] == -(s_.sum() * 2.0 ** 100)

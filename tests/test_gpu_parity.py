@@ -1128,3 +1128,40 @@ def test_infinite_pivots_in_warp_subtrees(precision):
         spchol.batch_solve(h, X, [M.n for M in mats], [1] * len(mats))
         assert all(np.isfinite(x).all() for x in X) and all(X[t][c, 0] == 0.0 for t, c in infinite)
     spchol.destroy(h)
+
+
+def test_pivot_square_roots_over_their_range():
+    # A diagonal matrix is one pivot a panel: l = d * r and x = r (r 1) with r
+    # the diagonal task's 1 / sqrt(d).  r keeps 57 bits before its rounding
+    # to nearest, so it is within 0.52 2^-52 of exact relative to a mantissa
+    # near 1, the worst case; l and x add half a unit of 2^-52 a product.  All
+    # exponents of the fast path, those on either side of it, mantissas at
+    # the ends of the range and random ones; and in the fallback's range
+    # the ends of FP64's (a subnormal, an infinite pivot: its root is
+    # infinite, and its unknown zero).
+    rng = np.random.default_rng(3)
+    e = np.arange(-123, 124)
+    m = np.concatenate([1.0 + np.array([0, 1, 2, 3, 2 ** 51, 2 ** 52 - 2, 2 ** 52 - 1]) * 2.0 ** -52,
+                        rng.uniform(1.0, 2.0, 193), 1.0 + rng.integers(0, 64, 20) * 2.0 ** -52])
+    d = (m[None, :] * 2.0 ** e[:, None].astype(float)).ravel()
+    d = np.concatenate([d, [5e-324, 2.0 ** -1060 * 3, 2.0 ** -1022, 1e-300, 1e300, np.finfo(float).max, np.inf]])
+    n = len(d)
+    s = spchol.SparseCholesky(n, np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32))
+    assert s.factorize(d) == 0
+    Lp, Li, Lx, perm = s.export_factor()
+    l = np.empty(n)
+    l[perm] = Lx
+    assert l[-1] == np.inf
+    with np.errstate(all="ignore"):
+        root = np.sqrt(d[:-1].astype(np.longdouble))
+        fast = np.abs(e).repeat(len(m)) <= 118
+        fast = np.concatenate([fast, np.zeros(6, bool)])
+        # the fallback divides by a rounded square root: one rounding more
+        err = np.abs(l[:-1] / root - 1) * 2.0 ** 52
+        assert err[fast].max() <= 1.1 and err.max() <= 1.6
+        x = s.solve(np.ones((n, 1), order="F"))[:, 0]
+        assert x[-1] == 0.0
+        near = (d[:-1] < 1e300) & (d[:-1] > 1e-300)
+        err = np.abs(x[:-1] * d[:-1].astype(np.longdouble) - 1)[near] * 2.0 ** 52
+        assert err[fast[near]].max() <= 1.6 and err.max() <= 2.6
+    s.close()
