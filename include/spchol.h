@@ -87,8 +87,9 @@ typedef struct spchol_options {
                              1..128 (1..64 with the tensor-core precisions), default 64 */
   int relax_zeros;        /* amalgamation: a child supernode is merged into its parent when every
                              merged column gains at most this many explicit zeros; default 4, 0 = off */
-  int tile_rows;          /* rows per update tile, 1..64; 0 = default (64).  The tensor-core tiles
-                             ignore it: 128 rows for TF32, 64 for SPCHOL_FP64_TC */
+  int tile_rows;          /* most rows per update tile, 1..64; 0 = default (64): a level of the panel
+                             tree with too few tiles for the GPU takes 32 or 16.  The tensor-core
+                             tiles ignore it: 128 rows for TF32, 64 for SPCHOL_FP64_TC */
   int ctas_per_sm;        /* persistent-kernel CTAs per SM; 0 = as many as fit */
   int deterministic;      /* 1: the static (target, source) order of Section IV-B: the update tiles
                              into each target panel, and the solve tiles into each panel's
@@ -158,7 +159,8 @@ typedef struct spchol_options {
                              x_s -= W^T x_below, with no diagonal solve between two steps of the
                              chain.  Costs the W buffer (the footprint counts it) and
                              2 (rows below) w^2 flops per such panel in the factorization.
-                             0 = default (64 for spchol_analyze, none for spchol_batch_analyze);
+                             0 = default (64 for spchol_analyze, or 32 where the device memory
+                             does not hold what 64 levels need; none for spchol_batch_analyze);
                              -1 = none; not used with deterministic != 0 */
 } spchol_options;
 
@@ -318,8 +320,9 @@ int spchol_export_factor(spchol_handle_t h, int64_t* nnz, int64_t* Lp, int64_t* 
  * device-clock start and end (ns, %globaltimer) of task i, in the task
  * numbering of the launch (factorization: diagonal tasks, then panel-solve
  * tiles, then update tiles, then subtree tasks, then the fan-in mode's gather
- * tasks; a task that never runs on its own -- a panel inside a subtree task --
- * reads 0 / 0).  Query form: out = NULL sets *count to the number of tasks.
+ * tasks; a task that never runs on its own -- of a panel inside a subtree task,
+ * or the panel-solve tile of a narrow panel of a small problem, whose diagonal
+ * task solves the rows below it -- reads 0 / 0).  Query form: out = NULL sets *count to the number of tasks.
  * Returns 0, -2 for a bad `which`, SPCHOL_ESTATE if not traced.
  */
 int spchol_trace_get(spchol_handle_t h, int which, uint64_t* out, int64_t* count);

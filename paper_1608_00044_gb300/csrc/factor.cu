@@ -444,7 +444,7 @@ __device__ void task_potrf(const FactorArgs& a, int s, double* sm, FactorShared&
   bool ok = true;
   const bool fuse = FUSE && fused_panel(a, s, w);
   if (!skip) {
-    stage_lower<true>(P, w, ld, sm);  // lower triangle; zeros above (used below for L11^{-1})
+    stage_lower<true>(P, w, ld, sm);  // lower triangle (what is above it is not read before L11^{-1} goes there)
     if (tid == 0) sh.flag = 0;  // 1: a failed pivot, whose columns are not used (a word of the CTA's own: the
                                 // status word is a trip to L2 ahead of the release)
     const int uw = warp == 3 ? kUpdWarps - 1 : warp > 3 ? warp - 1 : warp;  // number among the update warps
@@ -668,8 +668,10 @@ __device__ void task_trsm(const FactorArgs& a, int s, int k, double* smd, Factor
 template <bool FAN>
 __device__ __forceinline__ void target_update_done(const FactorArgs& a, int t, FactorShared& sh, bool release) {
   if constexpr (!FAN) {
-    // the diagonal task follows in this CTA, unless it holds a claimed slot
-    // whose task another would then wait for
+    // the diagonal task follows in this CTA, unless it holds a claimed slot of
+    // the high-priority ring or is inside a subtree task.  (A claimed slot of
+    // the other ring, or a stashed tile, waits for the diagonal task, as it
+    // would behind it in the rings.)
     if (release && threadIdx.x == 0 && count_down(&a.dep_f[t])) {
       if (sh.hold)
         ring2_push_one(rings_of(a), true, t);

@@ -21,7 +21,7 @@ constexpr int kFp64TcMinWidth = 16;
 // factorization and one solve.
 constexpr int kWDepth = 64;
 // Where the device memory does not hold that many levels' W (by 64^3 66 MB
-// beside a factor of 1.3 GB, but by 40^3 83 beside 171 and by 31^3 55 beside 58;
+// beside a factor of 1.3 GB, but by 40^3 83 beside 171 and by 31^3 51 beside 58;
 // 32 levels take 17 MB of all three): the next depth an analysis takes.
 constexpr int kWDepthLow = 32;
 

@@ -32,7 +32,7 @@ struct PlanParams {
   int top_depth = 128;
   // Rows per update tile: the panels of one level (distance to the root) take
   // the largest of tile_rows, 32 and 16 that still gives the level level_tiles
-  // tiles per resident CTA of the GPU (kPlanCtas); rows per panel-solve tile:
+  // tiles per CTA (kPlanCtas); rows per panel-solve tile:
   // of trsm_rows, 32 and 16, level_trsm tiles.  A level with fewer is on the
   // critical path and its tiles have to spread; one with more only pays each
   // tile's claim, staging and publishing.  level_tiles 0: by the size of the
@@ -82,7 +82,12 @@ struct PlanParams {
   int w_depth = 0;
 };
 
-// Resident CTAs of the factorization the plan is laid out for: 152 SMs x 5.
+// The CTAs that tile rows and the subtree cut are laid out for, a nominal unit:
+// 152 SMs x 5, the resident CTAs of the plain FP64 kernel.  FP32 panels run 6
+// per SM, the fan-in kernels 4, FP64_TC 3, TF32 2, and ctas_per_sm can lower
+// them; the limits below were measured against this unit in each mode, and with
+// ctas_per_sm 1 and 2 (31^3 FP64: factorization 24.2 -> 17.4 and 18.6 -> 11.1
+// ms, the rules before -> these).
 constexpr int kPlanCtas = 152 * 5;
 
 // In a small problem (at most kFuseFlops), a panel of at most kFuseWidth columns
@@ -306,7 +311,7 @@ inline const std::vector<FanEnt>& gather_entries(const Plan& P) { return P.gat_e
 constexpr int64_t kGatherValues = 8192;
 void split_gathers(Plan& plan, int64_t max_values);
 
-// The GPU launch's max_steps: a CTA's average share of all steps (kPlanCtas)
+// The GPU launch's max_steps: a CTA's average share of all steps (of kPlanCtas)
 // over kSubtreeShare.  A subtree task runs its steps one after
 // another, so one that holds more than the average share of the whole
 // factorization outlasts everything else: the 1e6-flop budget alone left the

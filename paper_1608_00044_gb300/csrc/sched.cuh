@@ -29,7 +29,9 @@ namespace spchol {
 // takes a visible high-priority task first.  A CTA claims a slot only when the
 // ring shows an unclaimed filled or reserved slot, so it holds a claimed slot
 // that is still empty only after losing a race for the last one, and a ready
-// task never waits behind a busy CTA for longer than such a race.  Every
+// task never waits behind a busy CTA for longer than such a race.  (With
+// tickets, see ring2_claim, an idle CTA takes its next slot of the
+// high-priority ring before the push, and waits for that slot alone.)  Every
 // claimed slot is filled eventually (a pusher reserves slots in order, so the
 // lowest claimed empty slot is the next to be filled).  A CTA holding a
 // claimed empty slot below the tail waits for the push that is filling it; one

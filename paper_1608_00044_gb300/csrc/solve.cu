@@ -1009,20 +1009,15 @@ __device__ __forceinline__ void release_tiles(const Ring2& q, const int32_t* lis
 }
 
 // Thread-level: every forward tile into W panel t has landed, so all of t's
-// forward tiles are ready (they read b_t); the first (the rows of the etree
-// parent, the next step of the chain) becomes the continuation if next is
-// given and free, the others go to the high-priority ring in one reservation.
-__device__ __forceinline__ void release_w_forward(const Ring2& q, const SolveArgs& a, int t, int* next) {
-  int first = a.pv.ns + a.st_first[t], count = a.nst[t];
-  if (next != nullptr && atomicCAS(next, -1, first) == -1) {
-    ++first;
-    --count;
-  }
-  ring2_push_span(q, true, first, count);
+// forward tiles are ready (they read b_t): pushed in one reservation.
+__device__ __forceinline__ void release_w_forward(const Ring2& q, const SolveArgs& a, int t) {
+  ring2_push_span(q, true, a.pv.ns + a.st_first[t], a.nst[t]);
 }
 
 // The same by the whole CTA, after a barrier: a panel near the root has more
 // than a hundred tiles, whose slots one thread would store one after another.
+// The first (the rows of the etree parent, the next step of the chain) becomes
+// the CTA's continuation if it holds no slot and has none yet.
 __device__ __forceinline__ void release_w_forward_cta(const Ring2& q, const SolveArgs& a, int t, SolveShared& sh) {
   const int first = a.pv.ns + a.st_first[t];
   if (threadIdx.x == 0) {
@@ -1135,7 +1130,7 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
             if (k < kWReady)
               sh.wl[k] = t;
             else
-              release_w_forward(q, a, t, nullptr);
+              release_w_forward(q, a, t);
           } else {
             keep_or_push(q, sh.hold ? nullptr : &sh.next, t);
           }
@@ -1226,7 +1221,9 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
 // kWsCap bytes -- are copied to shared memory while the current one is used;
 // only the right-hand sides' own trips to L2 are left on the chain.  Launches
 // over the 512 grids, one right-hand side, before -> now: forward 1.12 -> 0.74
-// ms (FP32 panels 1.17 -> 0.92), backward 1.05 -> 0.89 ms (1.52 -> 0.99).
+// ms (FP32 panels 1.17 -> 0.92), backward 1.05 -> 0.89 ms (1.52 -> 0.99) with 8
+// lanes an output (both launches and the task loop 2.37 -> 2.25 ms since they go by
+// the outputs, see there).
 constexpr int kWsWarps = 4;   // warps per CTA of the subtree solve launches
 constexpr int kWsNrc = 8;     // right-hand sides per pass (a panel is at most 32 wide)
 constexpr int kWsCap = 2048;  // bytes of a panel's operands in shared memory, two of them per warp (3072: no faster)
@@ -1399,7 +1396,7 @@ __device__ void subtree_forward(const SolveArgs& a, int k, unsigned char* buf, d
         const int t = a.st_tgt[e];
         if (t > hi && count_down(&a.fdep[t])) {
           if (is_wpanel(a, t))
-            release_w_forward(q, a, t, nullptr);
+            release_w_forward(q, a, t);
           else
             ring2_push_one(q, true, t);
         }

@@ -295,7 +295,7 @@ def test_torch_allocator_batch_handle():
 
 
 def test_memory_for_fewer_w_panels_is_enough():
-    # The default keeps W panels for 64 levels, 5.7 MB more than 32 levels do on
+    # The default keeps W panels for 64 levels, 4.8 MB more than 32 levels do on
     # a 24^3 Laplacian: an allocator that holds the smaller footprint and
     # half of the difference gets a handle (with 32 levels), one that holds
     # less than that ENOMEM, and a depth that the caller gives is not lowered.
