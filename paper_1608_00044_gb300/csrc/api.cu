@@ -1008,6 +1008,7 @@ int solve_permuted(spchol_handle_t h, double* Y, int nrhs, cudaStream_t st) {
   a.wbuf = h->d_wbuf;
   a.woff = P.n_wpan > 0 ? h->d_woff : nullptr;
   a.n_wpan = P.n_wpan;
+  a.chain = P.ns < 2 * P.levels;
   a.sub_lo = h->d_sub_lo;
   a.sub_hi = h->d_sub_hi;
   a.wsub = h->d_wsub;
@@ -1466,6 +1467,7 @@ int spchol_solve_noalloc(spchol_handle_t h, double* B, int64_t ldb, int nrhs, vo
   a.wbuf = h->d_wbuf;
   a.woff = P.n_wpan > 0 ? h->d_woff : nullptr;
   a.n_wpan = P.n_wpan;
+  a.chain = P.ns < 2 * P.levels;
   a.sub_lo = h->d_sub_lo;
   a.sub_hi = h->d_sub_hi;
   a.wsub = h->d_wsub;

@@ -136,6 +136,7 @@ struct SolveArgs {
   const void* wbuf;      // W = L21 L11^{-1} of the W panels (Plan::woff)
   const int64_t* woff;   // null: no W panels
   int32_t n_wpan;        // W panels: their backward diagonal tasks never run
+  int32_t chain;         // 1: a chain of panels, fewer than two to a level of the panel tree
   // The subtree tasks the factorization ran on single warps (FactorArgs::wsub),
   // solved by single warps too: their forward solves in a launch before the
   // task loop, their backward solves in one after it (subtree_solve_kernel).

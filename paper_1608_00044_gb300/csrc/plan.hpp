@@ -209,6 +209,7 @@ struct Plan {
   std::vector<int64_t> woff;
   int64_t n_w = 0;      // elements of the W buffer
   int32_t n_wpan = 0;   // W panels (backward diagonal tasks that never run)
+  int32_t levels = 0;   // of the panel tree
 
   // Deterministic order (params.deterministic; empty otherwise).  The update
   // tiles into each target panel form a chain in (source panel, row tile)

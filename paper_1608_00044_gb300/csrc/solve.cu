@@ -1059,15 +1059,16 @@ __global__ void __launch_bounds__(kSolveThreads, TC ? 4 : 5) solve_kernel(SolveA
         sh.next = -1;
       } else {
         int lo_ready;
-        // tickets while a task is one pass over the right-hand sides: then
-        // latency counts.  They hand the tasks to the CTAs in the order these
-        // fell idle, several on one SM, and with more passes the SM's FP64
-        // pipes make those wait.  Solves without / with them, ms: 64^3, 1
-        // right-hand side 9.50 / 9.24, 8 13.86 / 13.78; 27-point 30^3, 4 1.18 / 1.11;
-        // 31^3, 1 1.54 / 1.49, 8 1.93 / 1.91, 33 4.98 / 5.06; a full matrix of order
-        // 1500, 1 0.47 / 0.47, 8 0.70 / 0.78 (0.82 before there were any), 16 1.09 /
-        // 1.29, 33 1.92 / 2.39.
-        sh.task = ring2_claim(q, pend, &lo_ready, a.ntask_done, nullptr, a.nrhs <= kSolveNRC);
+        // Tickets hand the tasks to the CTAs in the order these fell idle,
+        // several on one SM.  Where latency counts they help; the tasks of a
+        // chain that pass over their right-hand sides several times wait for
+        // their SM's FP64 pipes instead.  Solves without / with them, ms: 64^3, 1
+        // right-hand side 9.50 / 9.24, 8 13.86 / 13.78; 33 x 41 x 37, 16 4.08 /
+        // 4.00; 27-point 30^3, 4 1.18 / 1.11, 16 2.14 / 2.08; 31^3, 1 1.54 / 1.49,
+        // 8 1.93 / 1.91, 33 4.98 / 5.06.  Chains: a full matrix of order 1500, 1
+        // 0.47 / 0.47, 8 0.70 / 0.78 (0.82 before there were any), 16 1.09 / 1.29,
+        // 33 1.92 / 2.39; a band in the fan-in mode, 11 114.2 / 118.6.
+        sh.task = ring2_claim(q, pend, &lo_ready, a.ntask_done, nullptr, !a.chain || a.nrhs <= kSolveNRC);
       }
       // While this CTA holds a claimed slot whose task is not yet pushed, it
       // takes no continuation: it comes back for that task after this one.

@@ -394,7 +394,7 @@ int build_plan(int64_t n, const int64_t* colptr, const int32_t* rowind, const in
   // ---- rows per update and panel-solve tile, level by level (PlanParams::level_tiles)
   std::vector<int32_t> upd_rows, solve_rows;
   {
-    const int32_t levels = ns == 0 ? 0 : *std::max_element(depth.begin(), depth.end()) + 1;
+    const int32_t levels = P.levels = ns == 0 ? 0 : *std::max_element(depth.begin(), depth.end()) + 1;
     const int32_t ur[3] = {prm.tile_rows, std::min(32, prm.tile_rows), std::min(16, prm.tile_rows)};
     const int32_t tr[3] = {prm.trsm_rows, std::min(32, prm.trsm_rows), std::min(16, prm.trsm_rows)};
     std::vector<int64_t> nu(2 * (size_t)levels, 0), nt(2 * (size_t)levels, 0);
